@@ -248,7 +248,7 @@ __device__ __forceinline__ void edge_kind(const int (&edge)[4], int x, int y, in
 // (the last iterate is used).
 enum { kWallSet = 0, kWallNoRoot = 1, kWallNoConv = 2 };
 template <typename S, typename Real>
-__device__ int maxent_wall(Real (&f)[9], unsigned solid) {
+__device__ int maxent_wall_general(Real (&f)[9], unsigned solid) {
   // the normal scaled by 36 (the weights are 4/36 and 1/36): integers, so
   // which unknowns are tangent to it, and whether it cancels, is exact
   int mx = 0, my = 0;
@@ -375,6 +375,259 @@ __device__ int maxent_wall(Real (&f)[9], unsigned solid) {
   for (int i = 0; i < 9; ++i)
     if (neg & (1u << i)) f[i] = (Real)((S)w_of(i) * exp(g * -a[i] - (S)1));
   return conv ? kWallSet : kWallNoConv;
+}
+
+// Double-float arithmetic: an unevaluated pair hi + lo carrying about 48
+// significant bits on the FP32 pipe (Dekker's products by a fused
+// multiply-add, Knuth's two-sum).
+struct Df {
+  float hi, lo;
+};
+__device__ __forceinline__ Df df_norm(float p, float e) {  // |e| <= |p|
+  const float s = p + e;
+  return Df{s, e - (s - p)};
+}
+__device__ __forceinline__ Df df_mul(Df a, Df b) {
+  const float p = a.hi * b.hi;
+  return df_norm(p, fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, fmaf(a.hi, b.hi, -p))));
+}
+__device__ __forceinline__ Df df_mul(Df a, float b) {
+  const float p = a.hi * b;
+  return df_norm(p, fmaf(a.lo, b, fmaf(a.hi, b, -p)));
+}
+__device__ __forceinline__ Df df_add(Df a, Df b) {
+  const float s = a.hi + b.hi, bb = s - a.hi;
+  return df_norm(s, ((a.hi - (s - bb)) + (b.hi - bb)) + (a.lo + b.lo));
+}
+__host__ __device__ constexpr Df df_const(double v) { return Df{(float)v, (float)(v - (double)(float)v)}; }
+
+// The pore wall's equation as a polynomial.  With the normal scaled by 36 to
+// the integer vector m = (mx, my), every unknown's e_i.n is -d_i / |m| with an
+// integer d_i > 0, so with t = exp(gamma / |m|) the unknowns are
+// (w_i / e) t^d_i and zero flux asks for
+//     p(t) = sum 36 w_i d_i t^d_i = 36 e T,   T = sum_{others} (e_j.m) f_j,
+// whose coefficients are integers.  d_i takes four values only: A = |mx| and
+// B = |my| on the axes, A + B and |A - B| on the diagonals (each with at most
+// one unknown, or two diagonals at A when B = 0), all formed from t^min(A, B)
+// and t^|A - B|: no exponential and no logarithm but in the FP32 start.
+struct WallPoly {
+  int A, B;            // |mx|, |my| (at most 6)
+  float ka, kb, ks, kd;  // coefficients of t^A, t^B, t^(A+B), t^|A-B|
+};
+
+// Start of the root in FP32: Newton's method on the convex log p as a function
+// of x = log t (it converges from any start; one step when every exponent is
+// equal, as on a flat wall).  Returns t, or 0 if it did not converge.
+__device__ __forceinline__ float wall_start(const WallPoly& w, float C) {
+  const float a = (float)w.A, b = (float)w.B, s = a + b, d = fabsf(a - b);
+  const int mn = min(w.A, w.B), df = abs(w.A - w.B);
+  const float logC = logf(C);
+  const float k0 = (w.ka + w.kb) + (w.ks + w.kd);
+  float x = (logC - logf(k0)) * (k0 / (w.ka * a + w.kb * b + w.ks * s + w.kd * d));
+  for (int it = 0; it < 24; ++it) {
+    const float t = expf(x), t2 = t * t, t4 = t2 * t2;
+    const float q = ((mn & 1) ? t : 1.f) * ((mn & 2) ? t2 : 1.f) * ((mn & 4) ? t4 : 1.f);
+    const float r = ((df & 1) ? t : 1.f) * ((df & 2) ? t2 : 1.f) * ((df & 4) ? t4 : 1.f);
+    const float big = q * r;  // t^max(A, B)
+    // (a term without an unknown may overflow: it must not turn 0 into NaN)
+    const float pa = w.ka > 0.f ? w.ka * (w.A >= w.B ? big : q) : 0.f;
+    const float pb = w.kb > 0.f ? w.kb * (w.A >= w.B ? q : big) : 0.f;
+    const float ps = w.ks > 0.f ? w.ks * (big * q) : 0.f;
+    const float pd = w.kd > 0.f ? w.kd * r : 0.f;
+    const float p = (pa + pb) + (ps + pd);
+    const float dp = (pa * a + pb * b) + (ps * s + pd * d);
+    if (!(dp > 0.f) || !isfinite(dp)) return 0.f;
+    const float step = (logf(p) - logC) * (p / dp);
+    x -= step;
+    if (fabsf(step) <= 5e-7f * (1.f + fabsf(x))) return expf(x);
+  }
+  return 0.f;
+}
+
+// Values (w_i / e) t^d_i of the unknowns by exponent, for axis directions along
+// x and y and for diagonals with d = A + B and d = |A - B|.
+template <typename Real>
+struct WallValues {
+  Real a, b, s, d;
+};
+
+// FP32 populations: one evaluation of p in double-float at the FP32 start, one
+// Newton step from its residual.  The relative step delta of t is at most 4e-6
+// (else the evaluation is repeated at the stepped start), which leaves t within
+// (d - 1) / 2 delta^2 < 1e-10 and the unknowns within 1.1e-9 relative of the
+// root before their FP32 rounding.  Returns false if the start did not
+// converge.
+__device__ __forceinline__ bool wall_root(const WallPoly& w, Df T, WallValues<float>& v) {
+  constexpr Df k36e = df_const(36.0 * 2.71828182845904523536);
+  constexpr Df kAxis = df_const(1.0 / 9.0 * 0.36787944117144232160);
+  constexpr Df kDiag = df_const(1.0 / 36.0 * 0.36787944117144232160);
+  const Df C = df_mul(T, k36e);
+  float t = wall_start(w, C.hi);
+  if (!(t > 0.f)) return false;
+  const int mn = min(w.A, w.B), df = abs(w.A - w.B);
+  const float a = (float)w.A, b = (float)w.B, s = a + b, d = (float)df;
+  const Df one{1.f, 0.f};
+  for (int it = 0; it < 4; ++it) {
+    const Df t1{t, 0.f};
+    const Df t2 = df_mul(t1, t1), t4 = df_mul(t2, t2);
+    const Df q = df_mul(df_mul((mn & 2) ? t2 : one, (mn & 1) ? t : 1.f), (mn & 4) ? t4 : one);
+    const Df r = df_mul(df_mul((df & 2) ? t2 : one, (df & 1) ? t : 1.f), (df & 4) ? t4 : one);
+    const Df big = df_mul(q, r), all = df_mul(big, q);
+    const Df pa = w.A >= w.B ? big : q, pb = w.A >= w.B ? q : big;
+    const Df p = df_add(df_add(df_mul(pa, w.ka), df_mul(pb, w.kb)),
+                        df_add(df_mul(all, w.ks), df_mul(r, w.kd)));
+    const float dp = (w.ka * a * pa.hi + w.kb * b * pb.hi) + (w.ks * s * all.hi + w.kd * d * r.hi);
+    const float delta = ((C.hi - p.hi) + (C.lo - p.lo)) / dp;
+    if (!(fabsf(delta) <= 4e-6f)) {
+      t *= 1.f + delta;
+      if (!(t > 0.f) || !isfinite(t)) return false;
+      continue;
+    }
+    auto value = [&](Df pw, float e, Df k) {  // k pw (1 + delta)^e to second order
+      const float f = pw.hi * k.hi;
+      const float lo = fmaf(pw.hi, k.lo, fmaf(pw.lo, k.hi, fmaf(pw.hi, k.hi, -f)));
+      const float c = e * delta;
+      return f + fmaf(f, fmaf(0.5f * (c - delta), c, c), lo);
+    };
+    v.a = value(pa, a, kAxis);
+    v.b = value(pb, b, kAxis);
+    v.s = value(all, s, kDiag);
+    v.d = value(r, d, kDiag);
+    return true;
+  }
+  return false;
+}
+
+// FP64 populations: Newton's method on p in FP64 from the FP32 start; a step
+// under 1e-8 leaves the quadratic remainder below FP64 rounding.
+__device__ __forceinline__ bool wall_root(const WallPoly& w, double T, WallValues<double>& v) {
+  constexpr double kE = 2.71828182845904523536, kInvE = 0.36787944117144232160;
+  const double C = 36.0 * kE * T;
+  const float start = wall_start(w, (float)C);
+  if (!(start > 0.f)) return false;
+  double t = (double)start;
+  const int mn = min(w.A, w.B), df = abs(w.A - w.B);
+  const double ka = w.ka, kb = w.kb, ks = w.ks, kd = w.kd;
+  const double da = ka * w.A, db = kb * w.B, ds = ks * (w.A + w.B), dd = kd * df;
+  bool near = false;
+  for (int it = 0; it < 8; ++it) {
+    const double t2 = t * t, t4 = t2 * t2;
+    double q = (mn & 1) ? t : 1.0, r = (df & 1) ? t : 1.0;
+    if (mn & 2) q *= t2;
+    if (mn & 4) q *= t4;
+    if (df & 2) r *= t2;
+    if (df & 4) r *= t4;
+    const double big = q * r, all = big * q;
+    const double pa = w.A >= w.B ? big : q, pb = w.A >= w.B ? q : big;
+    if (near) {
+      v.a = w_of(1) * kInvE * pa;
+      v.b = w_of(1) * kInvE * pb;
+      v.s = w_of(5) * kInvE * all;
+      v.d = w_of(5) * kInvE * r;
+      return true;
+    }
+    const double p = (ka * pa + kb * pb) + (ks * all + kd * r);
+    const double dp = (da * pa + db * pb) + (ds * all + dd * r);
+    const double delta = (C - p) / dp;
+    t += t * delta;
+    if (!(t > 0.0)) return false;
+    near = fabs(delta) <= 1e-8;
+  }
+  return false;
+}
+
+// The wall solve of a step.  The FP64 solve takes the polynomial form: with
+// its exponentials in FP64 (1/64 of the FP32 rate on this part, and every warp
+// with one wall node pays for 32) the solve took nearly all of the step's time,
+// 480 us a step at 1200 x 900 with FP32 populations; with one double-float
+// evaluation on the FP32 pipe the step takes 26 us.  The general form, in
+// logarithms, takes over where T is outside 1e-24 .. 1e24 for FP32 populations
+// (there the low parts of the FP32 pairs or the powers of t leave FP32's
+// range), outside 1e-34 .. 1e34 for FP64 ones (the range of the FP32 start), or
+// where the start did not converge; it works on a copy of f, so that the usual
+// path keeps f in registers.
+template <typename S, typename Real>
+__device__ __noinline__ int maxent_wall_rare(Real* f, unsigned solid) {
+  Real g[9];
+#pragma unroll
+  for (int i = 0; i < 9; ++i) g[i] = f[i];
+  const int r = maxent_wall_general<S>(g, solid);
+#pragma unroll
+  for (int i = 0; i < 9; ++i) f[i] = g[i];
+  return r;
+}
+
+template <typename S, typename Real>
+__device__ __forceinline__ int maxent_wall(Real (&f)[9], unsigned solid) {
+  if constexpr (sizeof(S) == 4) {
+    return maxent_wall_general<S>(f, solid);
+  } else {
+    int mx = 0, my = 0;
+#pragma unroll
+    for (int i = 1; i < 9; ++i)
+      if (solid & (1u << i)) {
+        const int w36 = i >= 5 ? 1 : 4;
+        mx -= w36 * cx_of(i);
+        my -= w36 * cy_of(i);
+      }
+    if (mx == 0 && my == 0) return kWallSet;
+    WallPoly w{abs(mx), abs(my), 0.f, 0.f, 0.f, 0.f};
+    unsigned neg = 0u;
+    // T = sum_{others} (e_j.m) f_j: integer multiples of the populations,
+    // summed in FP64, or in double-float for FP32 populations
+    double T = 0.0;
+    float Th = 0.f, Tl = 0.f;
+#pragma unroll
+    for (int i = 1; i < 9; ++i) {
+      const int d = -(cx_of(i) * mx + cy_of(i) * my);
+      if (((solid >> i) & 1u) && d > 0) {
+        neg |= 1u << i;
+        if (i == 1 || i == 3) w.ka += (float)(4 * d);
+        else if (i == 2 || i == 4) w.kb += (float)(4 * d);
+        else if (d == w.A + w.B) w.ks += (float)d;
+        else w.kd += (float)d;
+      } else if constexpr (sizeof(Real) == 8) {
+        T -= (double)d * f[i];
+      } else {
+        const float p = (float)-d * f[i], e = fmaf((float)-d, f[i], -p);
+        const float s = Th + p, bb = s - Th;
+        Tl += ((Th - (s - bb)) + (p - bb)) + e;
+        Th = s;
+      }
+    }
+    if (!neg) return kWallSet;
+    const Df Td = df_norm(Th, Tl);
+    const Real size = sizeof(Real) == 8 ? (Real)T : (Real)Td.hi;
+    if (!(size > (Real)0)) {
+#pragma unroll
+      for (int i = 1; i < 9; ++i)
+        if (neg & (1u << i)) f[i] = (Real)0;
+      return size < (Real)0 ? kWallNoRoot : kWallSet;
+    }
+    WallValues<Real> v;
+    constexpr double kLow = sizeof(Real) == 8 ? 1e-34 : 1e-24;
+    bool ok = size > (Real)kLow && size < (Real)(1.0 / kLow);
+    if (ok) {
+      if constexpr (sizeof(Real) == 8) ok = wall_root(w, T, v);
+      else ok = wall_root(w, Td, v);
+    }
+    if (!ok) {
+      Real g[9];
+#pragma unroll
+      for (int i = 0; i < 9; ++i) g[i] = f[i];
+      const int r = maxent_wall_rare<S, Real>(g, solid);
+#pragma unroll
+      for (int i = 0; i < 9; ++i) f[i] = g[i];
+      return r;
+    }
+#pragma unroll
+    for (int i = 1; i < 9; ++i)
+      if (neg & (1u << i)) {
+        const int d = -(cx_of(i) * mx + cy_of(i) * my);
+        f[i] = i == 1 || i == 3 ? v.a : i == 2 || i == 4 ? v.b : d == w.A + w.B ? v.s : v.d;
+      }
+    return kWallSet;
+  }
 }
 
 }  // namespace lbm
