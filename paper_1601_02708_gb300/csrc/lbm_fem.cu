@@ -18,9 +18,11 @@
 // arrays of A = M + theta dt K and B = M - (1 - theta) dt K.  The rows of
 // Dirichlet and inactive nodes are the identity in A and zero in B.  Each step
 // solves A x = B d^n (+ prescribed values) by Jacobi-preconditioned
-// BiCGSTAB in FP64 inside one cooperative launch (grid-wide barriers between
-// the phases of an iteration, dot products folded in a fixed order, so the
-// result is deterministic); the host reads the outcome once per step.  A
+// BiCGSTAB in FP64 inside one cooperative launch, the host reading the outcome
+// once per step: by tiles held in shared memory where the mesh fits (about
+// 200,000 nodes, k_bicgstab_tile), else over the nodes in global memory with
+// grid-wide barriers between the phases (k_bicgstab).  Sums are the same in
+// every block and in every run.  A
 // solve starts from the last converged solution (the previous Schwarz
 // iterate inside Algorithm 1), else from d^n.
 #include <cuda_runtime.h>
@@ -374,207 +376,432 @@ __global__ void __launch_bounds__(kThreads) k_bicgstab(const Solve S) {
   }
 }
 
-// ---- the linear solve of a small system in one block -----------------------
-// The same preconditioned BiCGSTAB with its vectors in shared memory, for
-// systems of at most kSmallNodes nodes, run by one block.  One SM then does
-// all the FP64 work, at 1/64 of the FP32 rate on this part (an FP64 warp
-// instruction holds the SM's FP64 pipe for about 16 cycles), so the work
-// that is the same for every thread is done once: each warp folds its
-// threads' partial sums, thread 0 adds the warp sums in warp order and forms
-// the iteration's scalars (alpha, omega, beta), and the others read them
-// from shared memory.  The preconditioned vectors p invd and s invd are
-// formed once an iteration behind a barrier, where the cooperative solve
-// re-forms them at every neighbour to save grid barriers.
-constexpr int kSmallThreads = 256;
-constexpr long long kSmallNodes = 2048;
-constexpr int kSmallVecs = 9;  // x, r, rhat, p, v, s, t, p invd, s invd
+// ---- the linear solve with its vectors in shared memory ---------------------
+// The same preconditioned BiCGSTAB for systems whose nodes fit the SMs' shared
+// memory, one block and one tile of tw x th nodes per SM.  What bounds it is
+// the FP64 pipe (1/64 of the FP32 rate on this part: a warp instruction holds
+// the SM's for 16 cycles) and the latency of the sums over the grid, so:
+//  - a block keeps r, p, v, p invd, s invd, t and the operator's rows of its
+//    tile in shared memory, and r, p, v, t of the one-node ring around it too,
+//    updating the ring's entries itself (1.26 times the tile's work at 22 x 13
+//    nodes) instead of forming nine neighbours' values for every node;
+//  - only the nodes on a tile's border go through global memory, v after the
+//    first product and t after the second;
+//  - two sums over the grid an iteration instead of three: with t.s, t.t,
+//    rhat.s, rhat.t and s.s from the second one, rhat.r = rhat.s - omega rhat.t
+//    and r.r = s.s - 2 omega t.s + omega^2 t.t.  Where that difference cancels
+//    ten digits the two products are summed directly;
+//  - every value that crosses blocks carries its own tag (put_tagged): no
+//    barrier, counter or memory fence, one trip through L2 for a sum;
+//  - scalars are formed by one thread.
+// A step of a 400 x 100 mesh with 13 to 17 iterations took 640 us with the
+// cooperative solve above (which forms p and s of nine neighbours per node and
+// crosses three atomic barriers an iteration) and takes 220 us; one of 40 x 10
+// elements in a single block, bound by that SM's FP64 pipe, took 15 us an
+// iteration, now 9.  An iteration's time is the FP64 pipe's latency (about 200
+// cycles an operation) along its chains: 2 us of products, 2 us of scalars, and
+// about 5 us for the two exchanges.
+constexpr int kTileVals = 5;        // values an exchange carries at most
+constexpr int kTileSlot = 8;        // 16-byte words from block to block: one 128-byte line
+constexpr int kTileMaxBlocks = 256;  // at most eight per polling lane
+// 12 warps: one node a thread of the 286-node tiles of a 400 x 100 mesh and of
+// their rings (with 8 the few nodes left over cost a second pass)
+constexpr int kTileThreads = 384;
+constexpr unsigned long long kTileWaitNs = 2000000000ull;  // 2 s
 
-// Warp sums of two values into red[0][warp], red[1][warp].
-__device__ __forceinline__ void small_warp_sums(double a, double b, double (*red)[kSmallThreads / 32]) {
+struct Outcome {  // of one solve, in page-locked host memory
+  Scal sc;
+  int iters, status;
+};
+
+struct TileSolve {
+  const double* A;
+  const double* invd;
+  const double* B;
+  double* d;         // state: d^n in, d^{n+1} out
+  double* xw;        // the last converged solution
+  const int* fixed_id;
+  const double* fixed_val;
+  // [n] v and t on the tiles' borders, tagged (tpub: r before the first
+  // iteration).  A block writes v again only past the exchange that follows
+  // its neighbours' reads of it (the second product's; for t the next first
+  // product's), so a reader never misses its tag.
+  ulonglong2* vpub;
+  ulonglong2* tpub;
+  ulonglong2* slots;  // [2][blocks][kTileSlot] exchanged values
+  Outcome* out;
+  int nxn, nyn, tw, th, ntx;
+  unsigned epoch;    // tag of the solve's first exchange
+  double tol;
+  int max_iter, warm;
+};
+
+// Shared memory of a block, in doubles.
+__host__ __device__ constexpr size_t tile_doubles(int tw, int th) {
+  const size_t ring = (size_t)(tw + 2) * (th + 2), own = (size_t)tw * th;
+  return 7 * ring + 11 * own + kTileVals * kTileThreads + ring + own;
+}
+
+__device__ __forceinline__ unsigned long long tile_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
+// A double in memory that other blocks read while it is written: two 64-bit
+// words, each half of it beside the tag of the exchange it belongs to.  A
+// reader knows the value by its words alone, so no flag, counter or fence
+// stands between the blocks.
+__device__ __forceinline__ void put_tagged(ulonglong2* at, double v, unsigned tag) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const unsigned long long t = (unsigned long long)tag << 32;
+  asm volatile("st.volatile.global.v2.u64 [%0], {%1, %2};" ::"l"(at), "l"(t | (b & 0xFFFFFFFFull)),
+               "l"(t | (b >> 32))
+               : "memory");
+}
+// The values with this tag at n places (at most N), all loads of a round in
+// flight together; bounded, false when the wait expired.
+template <int N, class At>
+__device__ __forceinline__ bool get_tagged(At at, int n, unsigned tag, double (&v)[N]) {
+  unsigned long long t0 = 0;
+  for (int spins = 1;; ++spins) {
+    unsigned long long lo[N], hi[N];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    a += __shfl_down_sync(0xffffffffu, a, o);
-    b += __shfl_down_sync(0xffffffffu, b, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    red[0][threadIdx.x >> 5] = a;
-    red[1][threadIdx.x >> 5] = b;
+    for (int i = 0; i < N; ++i)
+      if (i < n)
+        asm volatile("ld.volatile.global.v2.u64 {%0, %1}, [%2];"
+                     : "=l"(lo[i]), "=l"(hi[i])
+                     : "l"(at(i))
+                     : "memory");
+    bool all = true;
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+      if (i < n) {
+        all = all && (unsigned)(lo[i] >> 32) == tag && (unsigned)(hi[i] >> 32) == tag;
+        v[i] = __longlong_as_double((long long)((lo[i] & 0xFFFFFFFFull) | (hi[i] << 32)));
+      } else {
+        v[i] = 0.0;
+      }
+    if (all) return true;
+    if ((spins & 255) == 0) {
+      const unsigned long long now = tile_ns();
+      if (t0 == 0) t0 = now;
+      if (now - t0 > kTileWaitNs) return false;
+    }
   }
 }
 
-__global__ void __launch_bounds__(kSmallThreads) k_bicgstab_small(const Solve S) {
-  extern __shared__ double sm[];
-  __shared__ double red[2][kSmallThreads / 32];
-  // broadcast of thread 0's scalars: alpha, omega, beta; and its verdict
-  __shared__ double bc[3];
-  __shared__ int stop;  // 0 go on, 1 converged, 2 broke down
-  constexpr int kW = kSmallThreads / 32;
-  const int n = (int)S.n, nxn = S.nxn, nyn = S.nyn;
-  double* x = sm;
-  double* r = sm + n;
-  double* rh = sm + 2 * n;
-  double* p = sm + 3 * n;
-  double* v = sm + 4 * n;
-  double* s = sm + 5 * n;
-  double* t = sm + 6 * n;
-  double* y = sm + 7 * n;  // p invd (and d^n in the prologue)
-  double* z = sm + 8 * n;  // s invd (and b in the prologue)
-  const int q0 = threadIdx.x;
-  const bool lead = threadIdx.x == 0;
-  // row q of M u for a vector u in shared memory
-  auto row = [&](const double* __restrict__ M, const double* u, int q) {
-    const int i = q % nxn, j = q / nxn;
-    double acc = 0.0;
+// Sum of a warp's 32 x N doubles (the first n of each lane), the same in every
+// lane.  An FP64 addition returns after about 200 cycles here, so a shuffle
+// tree of them is slow; integers are not: every value is rounded once to
+// 2^-53 of the largest one's power of two, and the integers are summed exactly
+// in any order (three limbs, one reduction instruction each).  The rounding is
+// no more than that of adding the values one by one in FP64.
+template <int N>
+__device__ __forceinline__ double warp_sum(const double (&a)[N], int n) {
+  static_assert(32 * N <= 512, "54-bit integers, 9 bits of headroom, a sign");
+  constexpr unsigned kFull = 0xffffffffu;
+  unsigned top = 0;
 #pragma unroll
-    for (int k = 0; k < 9; ++k) {
-      const int ii = i + k % 3 - 1, jj = j + k / 3 - 1;
-      if (ii < 0 || ii >= nxn || jj < 0 || jj >= nyn) continue;
-      acc += __ldg(M + (long long)k * n + q) * u[jj * nxn + ii];
+  for (int i = 0; i < N; ++i)
+    if (i < n) top = max(top, ((unsigned)__double2hiint(a[i]) >> 20) & 0x7ffu);
+  top = __reduce_max_sync(kFull, top);
+  if (top == 0u) return 0.0;  // zeros (or below the normal range)
+  if (top == 0x7ffu) return __longlong_as_double(0x7ff8000000000000ll);
+  long long s = 0;
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+    if (i < n) {
+      const long long b = __double_as_longlong(a[i]);
+      const int e = (int)((b >> 52) & 0x7ff), sh = (int)top - e;
+      long long m = ((b & 0xFFFFFFFFFFFFFll) | 0x10000000000000ll) << 1;
+      m = (e == 0 || sh > 54) ? 0 : (m + ((1ll << sh) >> 1)) >> sh;
+      s += b < 0 ? -m : m;
     }
-    return acc;
-  };
-  for (int q = q0; q < n; q += kSmallThreads) y[q] = S.d[q];
+  const unsigned lo = __reduce_add_sync(kFull, (unsigned)s & 0x3FFFFFFu);
+  const unsigned mid = __reduce_add_sync(kFull, (unsigned)(s >> 26) & 0x3FFFFFFu);
+  const int hi = __reduce_add_sync(kFull, (int)(s >> 52));
+  const long long S = ((long long)hi << 52) + ((long long)mid << 26) + (long long)lo;
+  // value = S 2^(top - 1023 - 53)
+  if (top <= 64u) return ldexp((double)S, (int)top - 1076);
+  return (double)S * __longlong_as_double((long long)(top - 53u) << 52);
+}
+
+// Sums of V values over the threads of every block, left in sums[V] (the same
+// in every block): warp k sums the block's value k, the first warp writes the
+// block's values to its slot, and warp k reads and sums every block's value k;
+// meanwhile the other warps fetch the ring's border values, pub[rnode] to
+// u[rpos].  A slot is a 128-byte line of its own, written by one instruction:
+// a line that is written several times while it is polled is fetched anew
+// after every write, and values arrived 2.4 to 4.6 us after the last block had
+// written (words of eight blocks in a line, or five writes to one line) instead
+// of 0.9.  Slots alternate between two sets: a block can write a set again only
+// after every block has read it, since the exchange between them needs them
+// all.  The caller synchronises before it reads sums or the ring; *dead is set
+// when a wait expired.
+template <int V>
+__device__ __forceinline__ void tile_exchange(const double (&v)[V], int active, ulonglong2* slots,
+                                              unsigned tag, double* red, double* sums, int* dead,
+                                              const ulonglong2* pub, const int* rnode,
+                                              const int* rpos, int nr, double* u) {
+  constexpr int kW = kTileThreads / 32, kB = kTileMaxBlocks / 32;
+  static_assert(V < kW, "a warp per value, and some for the ring");
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5, nb = (int)gridDim.x;
+  ulonglong2* set = slots + (size_t)(tag & 1u) * nb * kTileSlot;
+#pragma unroll
+  for (int k = 0; k < V; ++k) red[k * kTileThreads + t] = v[k];
   __syncthreads();
-  // right-hand side (prescribed rows: their values), initial guess
-  double bb = 0.0;
-  for (int q = q0; q < n; q += kSmallThreads) {
-    const int f = S.fixed_id[q];
-    double bv, xv;
-    if (f >= 0) {
-      bv = S.fixed_val[f];
-      xv = bv;
-    } else if (f == -2) {
-      bv = 0.0;
-      xv = 0.0;
+  if (w < V) {
+    double a[kW];
+#pragma unroll
+    for (int i = 0; i < kW; ++i) a[i] = red[w * kTileThreads + 32 * i + lane];
+    const double s = warp_sum(a, active);
+    if constexpr (V == 1) {
+      if (lane == 0) put_tagged(set + (size_t)blockIdx.x * kTileSlot, s, tag);
     } else {
-      bv = row(S.B, y, q);
-      xv = S.warm ? S.w.x[q] : y[q];
+      if (lane == 0) sums[w] = s;
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * V) : "memory");
+      if (w == 0 && lane < V) put_tagged(set + (size_t)blockIdx.x * kTileSlot + lane, sums[lane], tag);
+      if (w == 0) __syncwarp();
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * V) : "memory");  // sums is rewritten below
     }
-    z[q] = bv;
-    x[q] = xv;
-    if (f == -1) bb += bv * bv;
+    double g[kB];
+    if (!get_tagged([&](int i) { return set + (size_t)(lane + 32 * i) * kTileSlot + w; },
+                    (nb - lane + 31) / 32, tag, g))
+      *dead = 1;
+    __syncwarp();
+    const double total = warp_sum(g, (nb + 31) / 32);
+    if (lane == 0) sums[w] = total;
+  } else {
+    for (int e = t - 32 * V; e < nr; e += kTileThreads - 32 * V) {
+      double val[1];
+      if (!get_tagged([&](int) { return pub + rnode[e]; }, 1, tag, val)) *dead = 1;
+      u[rpos[e]] = val[0];
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kTileThreads) k_bicgstab_tile(const TileSolve S) {
+  extern __shared__ double sm[];
+  __shared__ double sums[kTileVals];
+  __shared__ double bc[3];  // alpha, omega, beta
+  // 0 go on, 1 converged, 2 broke down, 3 iteration limit, 4 sum again, 5 a wait expired
+  __shared__ int stop;
+  __shared__ int nring, dead;
+  const int nxn = S.nxn, nyn = S.nyn, ld = S.tw + 2, ring = ld * (S.th + 2), cap = S.tw * S.th;
+  const int x0 = (int)(blockIdx.x % S.ntx) * S.tw, y0 = (int)(blockIdx.x / S.ntx) * S.th;
+  const int ow = min(S.tw, nxn - x0), oh = min(S.th, nyn - y0), own = ow * oh;
+  const long long n = (long long)nxn * nyn;
+  const int tid = threadIdx.x;
+  const bool lead = tid == 0;
+  double* r = sm;            // ring arrays: [th + 2][ld]
+  double* p = r + ring;
+  double* v = p + ring;
+  double* t = v + ring;
+  double* y = t + ring;      // p invd (x before the first iteration)
+  double* z = y + ring;      // s invd
+  double* iv = z + ring;
+  double* A = iv + ring;     // [9][cap] the operator's rows of the tile
+  double* x = A + 9 * cap;
+  double* rhat = x + cap;
+  double* red = rhat + cap;  // [kTileVals][kTileThreads]
+  int* rpos = (int*)(red + kTileVals * kTileThreads);  // ring list: position, node
+  int* rnode = rpos + ring;
+  int* opos = rnode + ring;  // position of each own node, border flag in bit 30
+  int* onode = opos + cap;
+  constexpr int kBorder = 1 << 30;
+  unsigned tag = S.epoch;
+
+  if (lead) nring = dead = 0;
+  __syncthreads();
+  auto start = [&](long long g) {  // the solve's starting value at a node
+    const int f = S.fixed_id[g];
+    return f >= 0 ? S.fixed_val[f] : f == -2 ? 0.0 : S.warm ? S.xw[g] : S.d[g];
+  };
+  for (int c = tid; c < ring; c += kTileThreads) {
+    const int cj = c / ld, ci = c - cj * ld, gi = x0 + ci - 1, gj = y0 + cj - 1;
+    const bool in = ci <= ow + 1 && cj <= oh + 1 && gi >= 0 && gi < nxn && gj >= 0 && gj < nyn;
+    const bool mine = in && ci >= 1 && ci <= ow && cj >= 1 && cj <= oh;
+    const long long g = (long long)gj * nxn + gi;
+    r[c] = p[c] = v[c] = t[c] = z[c] = 0.0;
+    y[c] = in ? start(g) : 0.0;
+    iv[c] = in ? S.invd[g] : 0.0;
+    if (mine) {
+      const int q = (cj - 1) * ow + (ci - 1);
+      const bool edge = ci == 1 || ci == ow || cj == 1 || cj == oh;
+      opos[q] = c | (edge ? kBorder : 0);
+      onode[q] = (int)g;
+    } else if (in) {
+      const int e = atomicAdd(&nring, 1);
+      rpos[e] = c;
+      rnode[e] = (int)g;
+    }
+  }
+  for (int e = tid; e < 9 * own; e += kTileThreads) {
+    const int k = e / own, q = e - k * own, qj = q / ow, qi = q - qj * ow;
+    A[k * cap + q] = S.A[k * n + (long long)(y0 + qj) * nxn + x0 + qi];
   }
   __syncthreads();
-  // r = b - A x, rhat = r, p = r, v = 0
-  double rr = 0.0;
-  for (int q = q0; q < n; q += kSmallThreads) {
-    const double rq = z[q] - row(S.A, x, q);
-    r[q] = rq;
-    rh[q] = rq;
-    p[q] = rq;
-    v[q] = 0.0;
+  // row q of A u for a ring array u (entries off the mesh are zero)
+  auto row = [&](const double* u, int q, int c) {
+    double acc[3] = {0.0, 0.0, 0.0};  // three chains: an FP64 operation is slow to return
+#pragma unroll
+    for (int k = 0; k < 9; ++k) acc[k / 3] += A[k * cap + q] * u[c + (k / 3 - 1) * ld + (k % 3 - 1)];
+    return (acc[0] + acc[1]) + acc[2];
+  };
+  // right-hand side and first residual; the norm is that of the free rows
+  double bb = 0.0, rr = 0.0;
+  for (int q = tid; q < own; q += kTileThreads) {
+    const int c = opos[q] & ~kBorder, g = onode[q], f = S.fixed_id[g];
+    double bv;
+    if (f >= 0) bv = S.fixed_val[f];
+    else if (f == -2) bv = 0.0;
+    else {
+      bv = spmv_row(S.B, S.d, x0 + (c % ld) - 1, y0 + (c / ld) - 1, nxn, nyn, n);
+      bb += bv * bv;
+    }
+    const double rq = bv - row(y, q, c);
+    x[q] = y[c];
+    rhat[q] = rq;
+    r[c] = p[c] = rq;
+    if (opos[q] & kBorder) put_tagged(S.tpub + g, rq, tag);
     rr += rq * rq;
   }
-  small_warp_sums(bb, rr, red);
+  const int nr = nring;
+  const int active = min(kTileThreads, own + 31) / 32;  // warps that hold own nodes
+  {
+    const double val[2] = {bb, rr};
+    tile_exchange<2>(val, active, S.slots, tag, red, sums, &dead, S.tpub, rnode, rpos, nr, r);
+  }
   __syncthreads();
   // thread 0's state: norms, rho and the iteration count
-  double bnorm2 = 0.0, rnorm2 = 0.0, tol2 = 0.0, rho = 0.0;
+  double bnorm2 = 0.0, rnorm2 = 0.0, tol2 = 0.0, rho = 0.0, rv = 0.0;
   int it = 0;
   if (lead) {
-    for (int k = 0; k < kW; ++k) {
-      bnorm2 += red[0][k];
-      rnorm2 += red[1][k];
-    }
+    bnorm2 = sums[0];
+    rnorm2 = rho = sums[1];
     tol2 = S.tol * S.tol * bnorm2;
-    rho = rnorm2;
     bc[0] = bc[1] = bc[2] = 0.0;
-    stop = rnorm2 <= tol2 ? 1 : 0;
+    stop = dead ? 5 : rnorm2 <= tol2 ? 1 : S.max_iter <= 0 ? 3 : 0;
   }
   __syncthreads();
   while (!stop) {
+    ++tag;
+    // p = r + beta (p - omega v), on the ring too; y = p invd
     const double beta = bc[2], omega_old = bc[1];
-    for (int q = q0; q < n; q += kSmallThreads) {
-      const double pq = r[q] + beta * (p[q] - omega_old * v[q]);
-      p[q] = pq;
-      y[q] = pq * S.invd[q];
+    for (int c = tid; c < ring; c += kTileThreads) {
+      const double pc = next_dir(r[c], p[c], v[c], beta, omega_old);
+      p[c] = pc;
+      y[c] = pc * iv[c];
     }
     __syncthreads();
-    double d0 = 0.0;
-    for (int q = q0; q < n; q += kSmallThreads) {
-      const double vq = row(S.A, y, q);
-      v[q] = vq;
-      d0 += rh[q] * vq;
+    double dot[1] = {0.0};
+    for (int q = tid; q < own; q += kTileThreads) {
+      const int c = opos[q] & ~kBorder;
+      const double vq = row(y, q, c);
+      v[c] = vq;
+      if (opos[q] & kBorder) put_tagged(S.vpub + onode[q], vq, tag);
+      dot[0] += rhat[q] * vq;
     }
-    small_warp_sums(d0, 0.0, red);
-    __syncthreads();
-    if (lead) {
-      double sum = 0.0;
-      for (int k = 0; k < kW; ++k) sum += red[0][k];
-      if (sum == 0.0 || !isfinite(sum))
-        stop = 2;
-      else
-        bc[0] = rho / sum;
+    tile_exchange<1>(dot, active, S.slots, tag, red, sums, &dead, S.vpub, rnode, rpos, nr, v);
+    if (lead) {  // the thread that folded the sum
+      rv = sums[0];
+      if (rv == 0.0 || !isfinite(rv)) stop = 2;
+      else bc[0] = rho / rv;
     }
     __syncthreads();
     if (stop) break;
+    // s = r - alpha v (in place), z = s invd
     const double alpha = bc[0];
-    for (int q = q0; q < n; q += kSmallThreads) {
-      const double sq = r[q] - alpha * v[q];
-      s[q] = sq;
-      z[q] = sq * S.invd[q];
+    for (int c = tid; c < ring; c += kTileThreads) {
+      const double sc = r[c] - alpha * v[c];
+      r[c] = sc;
+      z[c] = sc * iv[c];
     }
     __syncthreads();
-    double ts = 0.0, tt = 0.0;
-    for (int q = q0; q < n; q += kSmallThreads) {
-      const double tq = row(S.A, z, q);
-      t[q] = tq;
-      ts += tq * s[q];
-      tt += tq * tq;
+    ++tag;
+    double d5[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    for (int q = tid; q < own; q += kTileThreads) {
+      const int c = opos[q] & ~kBorder;
+      const double tq = row(z, q, c), sq = r[c], hq = rhat[q];
+      t[c] = tq;
+      if (opos[q] & kBorder) put_tagged(S.tpub + onode[q], tq, tag);
+      x[q] += alpha * y[c];
+      d5[0] += tq * sq;
+      d5[1] += tq * tq;
+      d5[2] += hq * sq;
+      d5[3] += hq * tq;
+      d5[4] += sq * sq;
     }
-    small_warp_sums(ts, tt, red);
+    tile_exchange<5>(d5, active, S.slots, tag, red, sums, &dead, S.tpub, rnode, rpos, nr, t);
     __syncthreads();
-    if (lead) {
-      double a = 0.0, b = 0.0;
-      for (int k = 0; k < kW; ++k) {
-        a += red[0][k];
-        b += red[1][k];
+    // omega = t.s / t.t and beta = (rho_new / rho) (alpha / omega), where
+    // alpha / rho = 1 / (rhat.v): the two divisions run side by side, in lanes
+    // 0 and 1 of the first warp
+    double rho_new = 0.0, omega_l = 0.0, per_rho = 0.0;
+    auto verdict = [&]() {  // thread 0, after rho_new and rnorm2
+      ++it;
+      if (dead) stop = 5;
+      else if (rnorm2 <= tol2) stop = 1;
+      else if (rho_new == 0.0 || omega_l == 0.0 || !isfinite(rho_new)) stop = 2;
+      else if (it >= S.max_iter) stop = 3;
+      else {
+        stop = 0;
+        bc[2] = rho_new * per_rho;
       }
-      bc[1] = b > 0.0 ? a / b : 0.0;
+      rho = rho_new;
+    };
+    if (tid < 32) {
+      const double rv0 = __shfl_sync(0xffffffffu, rv, 0);
+      const double q = tid == 1 ? sums[1] / (sums[0] * rv0) : sums[0] / sums[1];
+      per_rho = __shfl_sync(0xffffffffu, q, 1);
+      omega_l = sums[1] > 0.0 ? q : 0.0;
+      if (lead) {
+        bc[1] = omega_l;
+        rho_new = sums[2] - omega_l * sums[3];
+        rnorm2 = sums[4] - omega_l * (2.0 * sums[0] - omega_l * sums[1]);
+        if (!(rnorm2 > 1e-10 * sums[4]) && sums[4] > 0.0) stop = 4;
+        else verdict();
+      }
     }
     __syncthreads();
     const double omega = bc[1];
-    double rhn = 0.0;
-    rr = 0.0;
-    for (int q = q0; q < n; q += kSmallThreads) {
-      x[q] += alpha * y[q] + omega * z[q];
-      const double rq = s[q] - omega * t[q];
-      r[q] = rq;
-      rhn += rh[q] * rq;
-      rr += rq * rq;
-    }
-    small_warp_sums(rhn, rr, red);
-    __syncthreads();
-    if (lead) {
-      double rho_new = 0.0;
-      rnorm2 = 0.0;
-      for (int k = 0; k < kW; ++k) {
-        rho_new += red[0][k];
-        rnorm2 += red[1][k];
+    for (int q = tid; q < own; q += kTileThreads) x[q] += omega * z[opos[q] & ~kBorder];
+    for (int c = tid; c < ring; c += kTileThreads) r[c] -= omega * t[c];
+    if (stop == 4) {  // (the same in every block: all hold the same sums)
+      __syncthreads();
+      double d2[2] = {0.0, 0.0};
+      for (int q = tid; q < own; q += kTileThreads) {
+        const double rq = r[opos[q] & ~kBorder];
+        d2[0] += rhat[q] * rq;
+        d2[1] += rq * rq;
       }
-      ++it;
-      if (rnorm2 <= tol2)
-        stop = 1;
-      else if (rho_new == 0.0 || omega == 0.0 || !isfinite(rho_new))
-        stop = 2;
-      else if (it >= S.max_iter)
-        stop = 3;
-      else
-        bc[2] = (rho_new / rho) * (alpha / omega);
-      rho = rho_new;
+      ++tag;
+      tile_exchange<2>(d2, active, S.slots, tag, red, sums, &dead, nullptr, rnode, rpos, 0, t);
+      __syncthreads();
+      if (lead) {
+        rho_new = sums[0];
+        rnorm2 = sums[1];
+        verdict();
+      }
+      __syncthreads();
     }
-    __syncthreads();
+  }
+  if (dead) {  // a wait expired (stop is 2 or 5 in this block)
+    if (lead) *(volatile int*)&S.out->status = 1;
+    return;
   }
   // the solution, and the warm start of the next solve
-  for (int q = q0; q < n; q += kSmallThreads) {
-    S.d[q] = x[q];
-    S.w.x[q] = x[q];
+  for (int q = tid; q < own; q += kTileThreads) {
+    S.d[onode[q]] = x[q];
+    S.xw[onode[q]] = x[q];
   }
-  if (lead) {
-    S.sc->bnorm2 = bnorm2;
-    S.sc->rnorm2 = rnorm2;
-    S.sc->done = stop == 1 ? 1 : 0;
-    S.sc->breakdown = stop == 2 ? 1 : 0;
-    *S.iters = it;
+  if (lead && blockIdx.x == 0) {
+    S.out->sc.bnorm2 = bnorm2;
+    S.out->sc.rnorm2 = rnorm2;
+    S.out->sc.done = stop == 1 ? 1 : 0;
+    S.out->sc.breakdown = stop == 2 ? 1 : 0;
+    S.out->iters = it;
   }
 }
 
@@ -620,8 +847,13 @@ struct lbm_fem {
   int* status = nullptr;
   int grid = 0;             // blocks of the cooperative solve (all resident)
   double* scratch = nullptr;  // staging of host points / results of lbm_fem_interpolate
-  void* pinned = nullptr;     // page-locked read-back of a solve's outcome
-  bool small = false;         // solved by k_bicgstab_small (n <= kSmallNodes)
+  Outcome* pinned = nullptr;  // page-locked outcome of a solve
+  // solve by tiles (k_bicgstab_tile): tile size, 0 where the mesh does not fit
+  int tw = 0, th = 0, tiles = 0;
+  size_t tile_smem = 0;
+  ulonglong2* tagged = nullptr;  // exchange slots [2][tiles][kTileSlot], then v and t [2][n]
+  size_t tagged_b = 0;
+  unsigned epoch = 1;           // tag of the next solve's first exchange
   size_t scratch_n = 0;
   int last_iters = 0;
   double last_resid = 0.0;
@@ -635,9 +867,39 @@ struct lbm_fem {
 
 namespace {
 
+// Tile of k_bicgstab_tile for the mesh: the one whose block does the least
+// FP64 work per iteration, in warp instructions (6 a ring entry and 26 an own
+// node, and about 80 + 6 (blocks / 32 + 5) for the sums), among those whose
+// blocks are at most one per SM and fit its shared memory.  Larger meshes keep
+// the cooperative solve over all nodes (tiles = 0).
+constexpr size_t kTileSmem = 200 * 1024;
+void pick_tile(lbm_fem* f, int sms) {
+  const int most = sms < kTileMaxBlocks ? sms : kTileMaxBlocks;
+  const int cap = (int)(kTileSmem / sizeof(double) / 18);  // no tile holds more nodes
+  long long best = -1;
+  f->tiles = 0;
+  if (f->n > (long long)most * cap) return;
+  for (int tw = 1; tw <= f->nxn && tw <= cap; ++tw)
+    for (int th = 1; th <= f->nyn && tw * th <= cap; ++th) {
+      const long long nb = (long long)((f->nxn + tw - 1) / tw) * ((f->nyn + th - 1) / th);
+      if (nb > most) continue;
+      const size_t smem = tile_doubles(tw, th) * sizeof(double);
+      if (smem > kTileSmem) continue;
+      const long long ring = ((tw + 2) * (th + 2) + 31) / 32, own = (tw * th + 31) / 32;
+      const long long cost = 6 * ring + 26 * own + 6 * ((nb + 31) / 32);
+      if (best < 0 || cost < best) {
+        best = cost;
+        f->tw = tw;
+        f->th = th;
+        f->tiles = (int)nb;
+        f->tile_smem = smem;
+      }
+    }
+}
+
 void fem_free(lbm_fem* f) {
   void* ptrs[] = {f->A, f->B, f->d, f->b, f->vecs, f->fixed_id, f->fixed_val, f->part,
-                  f->sc, f->iters, f->scratch, f->bar, f->status, f->invd};
+                  f->sc, f->iters, f->scratch, f->bar, f->status, f->invd, f->tagged};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (f->pinned) cudaFreeHost(f->pinned);
@@ -796,13 +1058,18 @@ lbm_status lbm_fem_init(lbm_fem** out, const lbm_fem_params* p, const uint8_t* e
     long long cap = (long long)sms * (per_sm < 2 ? per_sm : 2);
     if (cap > kFoldCap) cap = kFoldCap;  // partials one fold can take
     f->grid = (int)(need < cap ? need : cap);
-    f->small = n <= kSmallNodes;
-    if (f->small && e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_bicgstab_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)(kSmallVecs * kSmallNodes * sizeof(double)));
+    if (e == cudaSuccess) pick_tile(f, sms);
+    if (e == cudaSuccess && f->tiles > 0)
+      e = cudaFuncSetAttribute(k_bicgstab_tile, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)kTileSmem);
   }
   al((void**)&f->part, 4 * (size_t)(f->grid > 0 ? f->grid : 1) * sizeof(double));
-  if (e == cudaSuccess) e = cudaMallocHost(&f->pinned, 256);
+  if (e == cudaSuccess) e = cudaMallocHost((void**)&f->pinned, sizeof(Outcome));
+  if (f->tiles > 0) {
+    f->tagged_b = 2 * ((size_t)f->tiles * kTileSlot + (size_t)n) * sizeof(ulonglong2);
+    al((void**)&f->tagged, f->tagged_b);
+    if (e == cudaSuccess) e = cudaMemset(f->tagged, 0, f->tagged_b);
+  }
   al((void**)&f->sc, sizeof(Scal));
   al((void**)&f->iters, sizeof(int));
   al((void**)&f->bar, 2 * sizeof(unsigned));
@@ -828,45 +1095,61 @@ lbm_status lbm_fem_step(lbm_fem* f, const double* dir_values) {
   if (!f) return ctx_fail(LBM_ERR_ARG, "lbm_fem_step: null solver");
   if (f->n_dir > 0 && !dir_values) return ctx_fail(LBM_ERR_ARG, "lbm_fem_step: null values");
   cudaStream_t s = f->stream;
-  if (f->n_dir > 0)
-    FCK(cudaMemcpyAsync(f->fixed_val, dir_values, f->n_dir * sizeof(double), cudaMemcpyDefault, s));
-  Solve S;
-  S.A = f->A;
-  S.invd = f->invd;
-  S.B = f->B;
-  S.d = f->d;
-  S.fixed_id = f->fixed_id;
-  S.fixed_val = f->fixed_val;
-  S.b = f->b;
-  S.w = f->w;
-  S.part = f->part;
-  S.bar = f->bar;
-  S.status = f->status;
-  S.sc = f->sc;
-  S.iters = f->iters;
-  S.nxn = f->nxn;
-  S.nyn = f->nyn;
-  S.n = f->n;
-  S.tol = f->p.tol;
-  S.max_iter = f->p.max_iter;
-  S.warm = f->warm ? 1 : 0;
-  void* args[] = {&S};
-  if (f->small)
-    k_bicgstab_small<<<1, kSmallThreads, kSmallVecs * f->n * sizeof(double), s>>>(S);
-  else
+  const double* fixed = f->fixed_val;
+  if (f->n_dir > 0) {
+    if (ctx_on_device(dir_values)) fixed = dir_values;  // read in place: this call waits
+    else FCK(cudaMemcpyAsync(f->fixed_val, dir_values, f->n_dir * sizeof(double),
+                             cudaMemcpyHostToDevice, s));
+  }
+  Outcome& h = *f->pinned;
+  h = Outcome{};
+  if (f->tiles > 0) {
+    // a solve makes at most 3 exchanges an iteration and one before the first
+    const unsigned long long span = 3ull * (unsigned)f->p.max_iter + 8;
+    if (f->epoch + span > 0xFFFFFFFFull) {  // tags about to repeat: start over
+      FCK(cudaMemsetAsync(f->tagged, 0, f->tagged_b, s));
+      f->epoch = 1;
+    }
+    ulonglong2* pub = f->tagged + 2 * (size_t)f->tiles * kTileSlot;
+    TileSolve T{f->A, f->invd, f->B, f->d, f->w.x, f->fixed_id, fixed, pub, pub + f->n, f->tagged,
+                f->pinned, f->nxn, f->nyn, f->tw, f->th, (f->nxn + f->tw - 1) / f->tw, f->epoch,
+                f->p.tol, f->p.max_iter, f->warm ? 1 : 0};
+    f->epoch += (unsigned)(span < 0x7FFFFFFFull ? span : 0x7FFFFFFFull);
+    void* args[] = {&T};
+    FCK(cudaLaunchCooperativeKernel((const void*)k_bicgstab_tile, dim3(f->tiles), dim3(kTileThreads),
+                                    args, f->tile_smem, s));
+    FCK(cudaGetLastError());
+    FCK(cudaStreamSynchronize(s));
+  } else {
+    Solve S;
+    S.A = f->A;
+    S.invd = f->invd;
+    S.B = f->B;
+    S.d = f->d;
+    S.fixed_id = f->fixed_id;
+    S.fixed_val = fixed;
+    S.b = f->b;
+    S.w = f->w;
+    S.part = f->part;
+    S.bar = f->bar;
+    S.status = f->status;
+    S.sc = f->sc;
+    S.iters = f->iters;
+    S.nxn = f->nxn;
+    S.nyn = f->nyn;
+    S.n = f->n;
+    S.tol = f->p.tol;
+    S.max_iter = f->p.max_iter;
+    S.warm = f->warm ? 1 : 0;
+    void* args[] = {&S};
     FCK(cudaLaunchCooperativeKernel((const void*)k_bicgstab, dim3(f->grid), dim3(kThreads), args,
                                     0, s));
-  FCK(cudaGetLastError());
-  struct Outcome {
-    Scal sc;
-    int iters, status;
-  };
-  static_assert(sizeof(Outcome) <= 256, "the outcome fits its pinned read-back");
-  Outcome& h = *(Outcome*)f->pinned;
-  FCK(cudaMemcpyAsync(&h.sc, f->sc, sizeof(Scal), cudaMemcpyDeviceToHost, s));
-  FCK(cudaMemcpyAsync(&h.iters, f->iters, sizeof(int), cudaMemcpyDeviceToHost, s));
-  FCK(cudaMemcpyAsync(&h.status, f->status, sizeof(int), cudaMemcpyDeviceToHost, s));
-  FCK(cudaStreamSynchronize(s));
+    FCK(cudaGetLastError());
+    FCK(cudaMemcpyAsync(&h.sc, f->sc, sizeof(Scal), cudaMemcpyDeviceToHost, s));
+    FCK(cudaMemcpyAsync(&h.iters, f->iters, sizeof(int), cudaMemcpyDeviceToHost, s));
+    FCK(cudaMemcpyAsync(&h.status, f->status, sizeof(int), cudaMemcpyDeviceToHost, s));
+    FCK(cudaStreamSynchronize(s));
+  }
   f->last_iters = h.iters;
   f->last_resid = h.sc.bnorm2 > 0 ? std::sqrt(h.sc.rnorm2 / h.sc.bnorm2) : std::sqrt(h.sc.rnorm2);
   f->warm = !h.status && h.sc.done;
