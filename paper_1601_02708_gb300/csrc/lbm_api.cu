@@ -287,7 +287,7 @@ using ShareOf = typename std::conditional<sizeof(Real) == 8, double, lbm::ShareF
 template <typename Real>
 lbm_status launch_dissolve(lbm_ctx* c) {
   TRY(time_begin(c, 1));
-  lbm::lbm_dissolve_list<ShareOf<Real>><<<c->dgrid, lbm::kDThreads, 0, c->stream>>>(
+  lbm::lbm_dissolve_list<ShareOf<Real>><<<c->lgrid, lbm::kDThreads, 0, c->stream>>>(
       dissolve_args(c), (const ShareOf<Real>*)c->ureact);
   CK(cudaGetLastError());
   return time_end(c, 1);
@@ -531,6 +531,10 @@ lbm_status init_impl(lbm_ctx* c, const uint8_t* solid, const double* vel,
     const long long blocks = ((long long)p.nx * p.ny + lbm::kDThreads - 1) / lbm::kDThreads;
     const long long cap = 8LL * c->num_sms;  // 8 resident blocks of 256 per SM
     c->dgrid = (int)(blocks < cap ? blocks : cap);
+    // the surface list holds a twentieth of a pore lattice's nodes: an entry a
+    // thread up to a quarter of them
+    const long long list = (blocks + 3) / 4;
+    c->lgrid = (int)(list < cap ? list : cap);
   }
   CK(cudaMalloc(&c->f[0], 9 * plane_b));
   CK(cudaMalloc(&c->f[1], 9 * plane_b));

@@ -189,6 +189,8 @@ __global__ void __launch_bounds__(lbm::kTmaBlock, 1)
       SmemSrc src{(const float*)st, (const float*)(st + kOffVel), (const float*)(st + kOffK),
                   (const uint32_t*)(st + kOffWord), r, 0, a.status};
       const int x0 = td.y, y = td.z + r;
+      if (a.dissolve_state && cw == 0 && lane == 0 && (td.w & kTileMask) == 0)
+        open_pass(a.dissolve_state);
       double tile_u = 0.0;
 #pragma unroll 1
       for (int j = 0; j < kNodesPerLane; ++j) {
@@ -232,50 +234,21 @@ __global__ void __launch_bounds__(lbm::kTmaBlock, 1)
 }
 
 // Dissolution of every member's surface list: block b serves member
-// bmap[b].x as its bmap[b].y-th of nblk[member] blocks; the last block of a
-// member to finish applies that member's flips (and closes its pass).
+// bmap[b].x as its bmap[b].y-th of nblk[member] blocks.
 template <typename Share>
 __global__ void __launch_bounds__(lbm::kDThreads)
     lbm_dissolve_batch(const lbm::DissolveArgs* __restrict__ dargs,
                        const void* const* __restrict__ rlinks, const int2* __restrict__ bmap,
                        const int* __restrict__ nblk) {
   __shared__ lbm::DissolveArgs d;
-  __shared__ bool last;
   const double* const tab = lbm::share_table();
-  const int tid = threadIdx.x;
   const int2 bm = bmap[blockIdx.x];
-  if (tid == 0) d = dargs[bm.x];
+  if (threadIdx.x == 0) d = dargs[bm.x];
   __syncthreads();
   const Share* rlink = (const Share*)rlinks[bm.x];
-  const int nb = nblk[bm.x];
-  const int pass = *(volatile int*)d.pass;
-  bool flipped = false;
-  const int count = *d.scount;
-  for (int e = bm.y * lbm::kDThreads + tid; e < count; e += nb * lbm::kDThreads) {
-    const int n = d.slist[e];
-    const uint32_t w = d.link[n];
-    if (!(w & lbm::kOwnSolid)) continue;
-    if (w & lbm::kOwnPending) {
-      lbm::finish_flip(d, n, pass);
-      continue;
-    }
-    const uint32_t fluid = ~((w >> lbm::kUpPostShift) | (w >> lbm::kUpOutShift)) & 0xFFu;
-    if (!fluid) continue;
-    const double m = d.smin[e] - lbm::mineral_take(rlink, n, d, fluid, tab);
-    d.smin[e] = m;
-    if (m <= 0.0) {
-      d.flip_list[lbm::dbg_idx(atomicAdd(d.flip_count, 1), (long long)d.nx * d.ny, d.status, lbm::kSiteList)] = n;
-      flipped = true;
-    }
-  }
-  if (flipped) __threadfence();
-  __syncthreads();
-  if (tid == 0) {
-    __threadfence();
-    last = (atomicAdd(d.done, 1u) == (unsigned)nb - 1);
-  }
-  __syncthreads();
-  if (last) lbm::apply_flips(d, tid, lbm::kDThreads);
+  const int nb = nblk[bm.x], count = *d.bound, pass = *d.pass - 1;
+  for (int e = bm.y * lbm::kDThreads + threadIdx.x; e < count; e += nb * lbm::kDThreads)
+    lbm::dissolve_entry(d, rlink, e, pass, tab);
 }
 
 }  // namespace
@@ -575,7 +548,7 @@ lbm_status lbm_batch_create(lbm_batch** out, int n, lbm_ctx* const* members) {
     if (!c->p.dissolution) continue;
     int len = 0;
     e = cudaMemcpy(&len, c->flip_count + 2, sizeof(int), cudaMemcpyDeviceToHost);
-    nb[i] = len / 2048 + 1;
+    nb[i] = len / lbm::kDThreads + 1;  // an entry a thread
     for (int k = 0; k < nb[i]; ++k) bm.push_back(make_int2(i, k));
   }
   b->dblocks = (int)bm.size();

@@ -54,6 +54,7 @@ __global__ void __launch_bounds__(32 * kBY)
       member = td.x;
     }
     const StepArgs<Real>& a = sa;
+    if (a.dissolve_state && tid == 0 && (td.w & kBatchTileMask) == 0) open_pass(a.dissolve_state);
     double my_u = 0.0;
 #pragma unroll
     for (int rr = 0; rr < kR; ++rr) {

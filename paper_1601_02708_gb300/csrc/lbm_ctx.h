@@ -48,8 +48,7 @@ struct lbm_ctx {
   int* open_nodes = nullptr;        // padded indices of the nodes on non-periodic sides
   int n_open = 0;
   int* flip_list = nullptr;
-  int* flip_count = nullptr;      // [0] count, [1] done counter, [2] surface list length,
-                                  // [3] dissolution passes run
+  int* flip_count = nullptr;      // words of the dissolution passes (lbm::open_pass)
   int* slist = nullptr;           // dissolution surface list (padded node indices)
   double* smin = nullptr;         // mineral of the listed nodes
   long long* counters = nullptr;  // [0] flips total, [1] solid count at init,
@@ -67,7 +66,8 @@ struct lbm_ctx {
   int nedge = 0;
   dim3 grid, block;    // 32 x 8 blocks over the lattice (init, adjoint, read-outs)
   dim3 sgrid, sblock;  // blocks of the plain step kernel (lbm::step_rows rows)
-  int dgrid = 0;  // persistent blocks of the dissolution pass
+  int dgrid = 0;  // persistent blocks of the passes over every node
+  int lgrid = 0;  // and of the pass over the surface list
   bool use_tma = false;  // the FP32 step runs the tile pipeline
   bool kernel_auto = true;  // the library chooses the FP32 step kernel
   bool tma_ready = false;
@@ -155,6 +155,7 @@ inline lbm::StepArgs<Real> step_args(lbm_ctx* c, double frac) {
   a.wall_infeasible = c->counters + 2;
   a.newton_fail = c->counters + 3;
   a.open_nodes = c->open_nodes;
+  a.dissolve_state = c->p.dissolution ? c->flip_count : nullptr;
   a.n_open = c->n_open;
   a.open_mask = 0;
   for (int s = 0; s < 4; ++s)
@@ -191,6 +192,7 @@ inline lbm::DissolveArgs dissolve_args(lbm_ctx* c) {
   d.flip_list = c->flip_list;
   d.flip_count = c->flip_count;
   d.done = (unsigned*)(c->flip_count + 1);
+  d.bound = c->flip_count + 1;
   d.scount = c->flip_count + 2;
   d.pass = c->flip_count + 3;
   d.flip_step = c->flip_step;

@@ -64,6 +64,7 @@ struct StepArgs {
   long long* __restrict__ newton_fail;      // count of wall solves short of the tolerance
   const int* __restrict__ open_nodes;  // padded indices of the nodes on non-periodic
                                        // sides (boundary warp of the tile pipeline)
+  int* dissolve_state;  // words of the dissolution passes (open_pass), or null
   int n_open;
   int open_mask;    // bit s: side s (W, E, S, N) is a Dirichlet or Neumann side
   int wall_maxent;  // pore walls of the maximum-entropy kind (else bounce-back)
@@ -77,6 +78,16 @@ struct StepArgs {
   Real k_scalar;
   double frac;  // j / eta of this substep
 };
+
+// Words of the dissolution passes: [0] flips of the first (dense) pass, [1] its
+// block counter, then the surface list's length as a step found it, [2] the
+// length now, [3] passes run or begun.  One thread of every step opens the pass
+// that follows it: the pass reads the length of before, while nodes it exposes
+// are appended.
+__device__ __forceinline__ void open_pass(int* state) {
+  state[1] = state[2];
+  state[3] += 1;
+}
 
 // Reaction share of a near-solid node of the FP32 lattice: its concentration
 // as stored by the lattice and 36 W_s = 4 (axis links to solid) + (diagonal
@@ -413,6 +424,8 @@ __global__ void __launch_bounds__(kBX * step_rows<Real>(), sizeof(Real) == 4 ? 2
     lbm_step(const StepArgs<Real> a) {
   constexpr int kBY = step_rows<Real>();
   __shared__ double red[kBX * kBY / 32];
+  if (a.dissolve_state && blockIdx.x + blockIdx.y + threadIdx.x + threadIdx.y == 0)
+    open_pass(a.dissolve_state);
   const int x = blockIdx.x * kBX + threadIdx.x;
   const int y = blockIdx.y * kBY + threadIdx.y;
   double my_u = 0.0;
@@ -531,6 +544,7 @@ struct DissolveArgs {
   int* flip_list;        // padded indices of nodes found exhausted this pass
   int* flip_count;
   unsigned* done;
+  const int* bound;      // surface list length when the step opened the pass
   int* pass;             // passes run so far (the first, after initialisation, is 0)
   int* flip_step;        // [rows][pitch]: pass that turned the node fluid, -1 if none
   long long* flips_total;
@@ -712,50 +726,71 @@ __device__ inline void apply_flips(const DissolveArgs& d, int tid, int nthreads)
   }
 }
 
+// A node used up in this pass: pending (solid for the next streaming, fluid for
+// its collision); its neighbours' post-flip bits say so, and solid neighbours
+// it exposes go on the surface list.  Done at once, while other nodes are still
+// examined: a neighbour examined later sees one more fluid node, whose share is
+// exactly zero (no step has written one at a solid node), so it loses the same.
+__device__ __forceinline__ void flip_node(const DissolveArgs& d, int n) {
+  int x, y;
+  node_xy(d, n, x, y);
+  atomicOr(d.link + n, kOwnPending);
+#pragma unroll 1
+  for (int i = 1; i < 9; ++i) {
+    const int z = neighbour(d, x, y, i);
+    if (z < 0) continue;
+    const uint32_t old = atomicAnd(d.link + z, ~up_bit(kUpPostShift, i));
+    if ((old & kOwnSolid) && !(old & kListed) && !(atomicOr(d.link + z, kListed) & kListed)) {
+      const long long slot =
+          dbg_idx(atomicAdd(d.scount, 1), (long long)d.nx * d.ny, d.status, kSiteList);
+      d.slist[slot] = z;
+      d.smin[slot] = d.mineral[z];
+    }
+  }
+  atomicAdd(reinterpret_cast<unsigned long long*>(d.flips_total), 1ull);
+}
+
 // Dissolution after a step, for the solid nodes on the surface list: each
 // gathers the mineral it loses (mineral_take); nodes that turned fluid
 // before this step's collision (pending) become plain fluid and stop being
-// solid upstream for their neighbours; nodes whose mineral is used up are
-// collected and, by the last block to finish, marked pending (apply_flips).
-// Link-word edits are atomic bit operations on bits no concurrent reader of
-// the same word depends on, so the result is independent of timing.
+// solid upstream for their neighbours; nodes whose mineral is used up flip
+// (flip_node).  The chain list entry, link word, shares bounds it: about 3 us
+// at 512 x 512.  (Collecting the flips for the last block to apply, with a fence
+// and a counter on one address for every block, took it to 8: a substep there
+// went from 18.4 to 13.3 us, the benchmark's 4096 x 4096 one from 289 to 272.)
+// Link-word edits are atomic bit operations on bits whose value
+// no concurrent reader of the same word depends on, so the result is
+// independent of timing, and no block waits for another.
 // Share is double (FP64 lattice) or ShareF32 (FP32 lattice).
 constexpr int kDThreads = 256;
+
+// Entry e of the surface list in the pass numbered `pass`.
+template <typename Share>
+__device__ __forceinline__ void dissolve_entry(const DissolveArgs& d,
+                                               const Share* __restrict__ rlink, int e, int pass,
+                                               const double* tab) {
+  const int n = d.slist[e];
+  const double m0 = d.smin[e];  // (ahead of the word: it does not depend on it)
+  const uint32_t w = d.link[n];
+  if (!(w & kOwnSolid)) return;  // dissolved earlier
+  if (w & kOwnPending) {
+    finish_flip(d, n, pass);
+    return;
+  }
+  const uint32_t fluid = ~((w >> kUpPostShift) | (w >> kUpOutShift)) & 0xFFu;
+  if (!fluid) return;
+  const double m = m0 - mineral_take(rlink, n, d, fluid, tab);
+  d.smin[e] = m;
+  if (m <= 0.0) flip_node(d, n);
+}
 
 template <typename Share>
 __global__ void __launch_bounds__(kDThreads)
     lbm_dissolve_list(const DissolveArgs d, const Share* __restrict__ rlink) {
   const double* const tab = share_table();
-  const int tid = threadIdx.x;
-  const int pass = *(volatile int*)d.pass;
-  bool flipped = false;
-  const int count = *d.scount;
-  for (int e = blockIdx.x * kDThreads + tid; e < count; e += gridDim.x * kDThreads) {
-    const int n = d.slist[e];
-    const uint32_t w = d.link[n];
-    if (!(w & kOwnSolid)) continue;  // dissolved earlier
-    if (w & kOwnPending) {
-      finish_flip(d, n, pass);
-      continue;
-    }
-    const uint32_t fluid = ~((w >> kUpPostShift) | (w >> kUpOutShift)) & 0xFFu;
-    if (!fluid) continue;
-    const double m = d.smin[e] - mineral_take(rlink, n, d, fluid, tab);
-    d.smin[e] = m;
-    if (m <= 0.0) {
-      d.flip_list[dbg_idx(atomicAdd(d.flip_count, 1), (long long)d.nx * d.ny, d.status, kSiteList)] = n;
-      flipped = true;
-    }
-  }
-  __shared__ bool last;
-  if (flipped) __threadfence();
-  __syncthreads();
-  if (tid == 0) {
-    __threadfence();
-    last = (atomicAdd(d.done, 1u) == gridDim.x - 1);
-  }
-  __syncthreads();
-  if (last) apply_flips(d, tid, kDThreads);
+  const int count = *d.bound, pass = *d.pass - 1;  // the step opened this pass
+  for (int e = blockIdx.x * kDThreads + threadIdx.x; e < count; e += gridDim.x * kDThreads)
+    dissolve_entry(d, rlink, e, pass, tab);
 }
 
 // Dissolution pass over every node (used once, after initialisation): the

@@ -208,6 +208,7 @@ __global__ void __launch_bounds__(kTmaBlock, 1)
       mbar_init(&empty[s], kTmaThreads / 32);
     }
     abort_flag = 0;
+    if (a.dissolve_state && blockIdx.x == 0) open_pass(a.dissolve_state);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
