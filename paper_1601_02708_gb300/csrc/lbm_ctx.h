@@ -10,6 +10,24 @@
 #include "lbm_ade.h"
 #include "lbm_tma.cuh"
 
+// Launch as a programmatic dependent of the stream's last kernel (pdl_wait in
+// lbm_kernels.cuh); behind any other work it is an ordinary launch.
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                              cudaStream_t stream, const A&... args) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 struct DiagDev {
   double mass, J, flux;
   long long infeasible;

@@ -21,6 +21,19 @@
 
 namespace lbm {
 
+// A kernel launched as a programmatic dependent (launch_pdl) is set up on the SMs
+// while its predecessor's last blocks run.  pdl_wait returns once every earlier
+// kernel has completed and its writes are visible, and then lets the successor
+// be set up in turn; nothing before it may touch global memory.  Used where
+// one kernel of one block per SM follows itself in a stream (the pair's steps,
+// 31.4 -> 28.8 us at 1024 x 768).  Sequences with a kernel of many blocks, or
+// with local memory, lose by it (a dissolving 512 x 512 substep 13.3 -> 17.7
+// us), and replayed graphs gain nothing.
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;");
+}
+
 constexpr int kBX = 32;  // generic kernel: threads along x per block
 constexpr int kBY = 8;   // generic kernel: rows per block
 

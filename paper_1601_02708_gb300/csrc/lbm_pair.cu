@@ -72,6 +72,7 @@ __global__ void __launch_bounds__(kTmaBlock, 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
+  pdl_wait();
 
   double u0 = 0.0, u1 = 0.0;  // block's mass of each field
   if (warp == 0) {
@@ -283,11 +284,9 @@ lbm_status lbm_pair_substeps(lbm_pair* pr, int n, int eta, const double* a_dir_t
     s1.link = a->link;  // one geometry: field B reads field A's links and velocity
     s1.vel = (const float*)a->vel;
     const PairMaps& m = pr->maps[a->cur];
-    if (j == n)
-      lbm_step_tma_pair<true><<<pr->grid, kTmaBlock, kPSmem, a->stream>>>(s0, s1, m, pr->ntx, pr->nty);
-    else
-      lbm_step_tma_pair<false><<<pr->grid, kTmaBlock, kPSmem, a->stream>>>(s0, s1, m, pr->ntx, pr->nty);
-    const cudaError_t e = cudaGetLastError();
+    const cudaError_t e =
+        launch_pdl(j == n ? lbm_step_tma_pair<true> : lbm_step_tma_pair<false>, pr->grid, kTmaBlock,
+                   kPSmem, a->stream, s0, s1, m, pr->ntx, pr->nty);
     if (e != cudaSuccess) return ctx_fail(LBM_ERR_CUDA, "lbm_pair_substeps: %s", cudaGetErrorString(e));
     for (lbm_ctx* c : pr->c) {
       c->cur ^= 1;
