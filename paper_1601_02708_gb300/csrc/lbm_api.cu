@@ -1264,6 +1264,10 @@ lbm_status lbm_restore(lbm_ctx* c, const void* buf, size_t bytes) {
     CK(cudaMemcpyAsync(s[i].ptr, (const char*)buf + off, s[i].bytes, k, c->stream));
     off += align256(s[i].bytes);
   }
+  // the blob holds no shares (every step writes those of its fluid nodes), and
+  // a node that is solid again must not keep the one of its fluid life: a pass
+  // reads a zero there while the node flips (lbm::flip_node)
+  if (c->p.dissolution) CK(cudaMemsetAsync(c->ureact, 0, (size_t)c->plane * 8, c->stream));
   c->steps = h.steps;
   c->nparts = h.nparts;
   if (!dev) CK(cudaStreamSynchronize(c->stream));

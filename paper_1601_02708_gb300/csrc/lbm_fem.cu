@@ -1068,7 +1068,7 @@ lbm_status lbm_fem_init(lbm_fem** out, const lbm_fem_params* p, const uint8_t* e
   if (f->tiles > 0) {
     f->tagged_b = 2 * ((size_t)f->tiles * kTileSlot + (size_t)n) * sizeof(ulonglong2);
     al((void**)&f->tagged, f->tagged_b);
-    if (e == cudaSuccess) e = cudaMemset(f->tagged, 0, f->tagged_b);
+    if (e == cudaSuccess) e = cudaMemsetAsync(f->tagged, 0, f->tagged_b, f->stream);
   }
   al((void**)&f->sc, sizeof(Scal));
   al((void**)&f->iters, sizeof(int));

@@ -764,7 +764,8 @@ __device__ inline void apply_flips(const DissolveArgs& d, int tid, int nthreads)
 // its collision); its neighbours' post-flip bits say so, and solid neighbours
 // it exposes go on the surface list.  Done at once, while other nodes are still
 // examined: a neighbour examined later sees one more fluid node, whose share is
-// exactly zero (no step has written one at a solid node), so it loses the same.
+// exactly zero (no step has written one at a solid node, and a restored lattice
+// starts from zero shares), so it loses the same.
 __device__ __forceinline__ void flip_node(const DissolveArgs& d, int n) {
   int x, y;
   node_xy(d, n, x, y);

@@ -56,3 +56,33 @@ def test_many_flips_in_one_pass(oracle_mod, shape, edges, batch):
         assert np.abs(lat.mineral() - ahead.mineral())[left].max() <= 5e-14
         most, before = max(most, flips - before), flips
     assert most > 50
+
+
+@pytest.mark.parametrize("shape", [(33, 40), (400, 300)])
+@pytest.mark.parametrize("precision", [32, 64])
+def test_restored_solids_have_no_shares(oracle_mod, shape, precision):
+    """Nodes that were fluid, with shares, and are solid again after a restore
+    flip anew beside neighbours examined in the same pass: every run from the
+    restored state ends in the same bits, and the FP64 mask is the oracle's."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1601_02708_gb300 import LBM
+    nx, ny = shape
+    kw = _case(nx, ny, (1, 1, 1, 1))
+    ud = inputs.edge_array(nx, ny, 1.0, 1.0, 1.0, 1.0)
+    lat = LBM(nx, ny, 0.8, precision=precision, **kw)
+    start = lat.save()
+    n = 40
+    runs = []
+    for _ in range(6):
+        lat.restore(start)
+        lat.substeps(n, 1, ud, ud)
+        runs.append((lat.solid(), lat.mineral(), lat.flip_steps()))
+    assert lat.diagnostics()["flips"] > 200
+    for run in runs[1:]:
+        assert all(np.array_equal(a, b) for a, b in zip(run, runs[0]))
+    if precision == 64:
+        ref = oracle_mod.LBMOracle(nx, ny, 0.8, **kw)
+        ref.substeps(n, 1, ud, ud)
+        assert np.array_equal(runs[0][0], ref.solid())
