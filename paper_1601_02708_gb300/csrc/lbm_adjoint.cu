@@ -142,21 +142,57 @@ __device__ __forceinline__ void adjoint_node(const AdjArgs<Real>& a, int x, int 
     if (unknown) {
       int dside, nside, sx, sy;
       edge_kind(a.edge, x, y, a.nx, a.ny, &dside, &nside, &sx, &sy);
-      // t = sum_U w_i nu_i / W_U over the unknowns, in FP64 on either lattice
-      // (the transpose of the forward solves, which run in FP64)
-      double t = 0.0, wu = 0.0;
+      // t = sum_U w_i nu_i / W_U over the unknowns (the transpose of the forward
+      // solves): in double-float on the FP32 lattice where W_U is a side's or a
+      // corner's (lbm::maxent_dirichlet says why), else in FP64
+      const int c36 = set_weight36(unknown);
+      bool pair = sizeof(Real) == 4 && (c36 == 6 || c36 == 11);
+      double t = 0.0;
+      EdgeSum tp;
+      if (pair) {
+        float most = 0.f;
 #pragma unroll
-      for (int i = 0; i < 9; ++i)
-        if (unknown & (1u << i)) {
-          t += w_of(i) * (double)nu[i];
-          wu += w_of(i);
-        }
-      t /= wu;
+        for (int i = 1; i < 9; ++i)
+          if (unknown & (1u << i)) {
+            const float v = (i < 5 ? 4.f : 1.f) * (float)nu[i];
+            most = fmaxf(most, fabsf(v));
+            tp.add(v);
+          }
+        tp.norm();
+        pair = fabsf(tp.hi) <= most * 16.f && most < kEdgeHigh;  // (neither NaN nor infinite)
+        tp = edge_over(tp, c36);
+        t = (double)tp.hi + (double)tp.lo;
+      }
+      if (sizeof(Real) == 8 && (c36 == 6 || c36 == 11)) {
+        double v[9];
+#pragma unroll
+        for (int i = 1; i < 9; ++i) v[i] = unknown & (1u << i) ? (double)nu[i] : 0.0;
+        t = (4.0 * ((v[1] + v[2]) + (v[3] + v[4])) + ((v[5] + v[6]) + (v[7] + v[8]))) *
+            (c36 == 6 ? 1.0 / 6 : 1.0 / 11);
+      } else if (!pair) {
+        double wu = 0.0;
+#pragma unroll
+        for (int i = 0; i < 9; ++i)
+          if (unknown & (1u << i)) {
+            t += w_of(i) * (double)nu[i];
+            wu += w_of(i);
+          }
+        t /= wu;
+      }
+      // nu + d t, rounded once
+      auto plus_t = [&](Real v, int d) -> Real {
+        if (sizeof(Real) == 8 || !pair) return (Real)((double)v + d * t);
+        EdgeSum r;
+        r.hi = d * tp.hi;
+        r.lo = d * tp.lo;
+        r.add((float)v);
+        return (Real)__fadd_rn(r.hi, r.lo);
+      };
       if (dside >= 0) {
         const int slot = edge_slot(dside, x, y, a.nx, a.ny);
 #pragma unroll
         for (int i = 0; i < 9; ++i)
-          if (!(unknown & (1u << i))) nu[i] = (Real)((double)nu[i] - t);
+          if (!(unknown & (1u << i))) nu[i] = plus_t(nu[i], -1);
         atomicAdd(a.g_ua + slot, (1.0 - a.frac) * t);
         atomicAdd(a.g_ub + slot, a.frac * t);
       } else {
@@ -165,7 +201,7 @@ __device__ __forceinline__ void adjoint_node(const AdjArgs<Real>& a, int x, int 
 #pragma unroll
           for (int i = 0; i < 9; ++i) {
             const int d = cx_of(i) * sx + cy_of(i) * sy;
-            if (!(unknown & (1u << i)) && d != 0) nu[i] = (Real)((double)nu[i] + d * t);
+            if (!(unknown & (1u << i)) && d != 0) nu[i] = plus_t(nu[i], d);
           }
           atomicAdd(a.g_q + slot, -t);
         }
