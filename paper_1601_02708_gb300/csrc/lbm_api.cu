@@ -746,13 +746,7 @@ struct BlobHeader {
   int nx, ny, precision, dissolution, nparts, pad;
 };
 const unsigned long long kMagic = 0x4C424D4144453035ull;  // "LBMADE05"
-static_assert(sizeof(BlobHeader) <= 64, "the header fits its pinned read-back slot");
-
-// Write a blob header into device memory byte by byte (any alignment).
-__global__ void k_put_blob_header(unsigned char* dst, const BlobHeader h) {
-  const unsigned char* src = reinterpret_cast<const unsigned char*>(&h);
-  for (int i = threadIdx.x; i < (int)sizeof(BlobHeader); i += blockDim.x) dst[i] = src[i];
-}
+static_assert(sizeof(BlobHeader) <= 64 && sizeof(BlobHeader) <= kCopyHead, "the header fits its pinned read-back slot");
 
 // Copy a padded device field out to a caller array (host or device) of
 // `planes` [ny][nx] planes, converting to O.
@@ -793,17 +787,22 @@ bool ctx_on_device(const void* p) { return on_device(p); }
 
 lbm_status ctx_stage_edges(lbm_ctx* c, const double* ua, const double* ub, const double* q) {
   const size_t eb = (size_t)c->nedge * sizeof(double);
-  double* e = c->edge;
-  if (ua) CK(cudaMemcpyAsync(e, ua, eb, kind_from(ua), c->stream));
-  else CK(cudaMemsetAsync(e, 0, eb, c->stream));
-  const double* b = ub ? ub : ua;
-  if (b) CK(cudaMemcpyAsync(e + c->nedge, b, eb, kind_from(b), c->stream));
-  else CK(cudaMemsetAsync(e + c->nedge, 0, eb, c->stream));
-  if (q) CK(cudaMemcpyAsync(e + 2 * c->nedge, q, eb, kind_from(q), c->stream));
-  else CK(cudaMemsetAsync(e + 2 * c->nedge, 0, eb, c->stream));
+  const double* src[3] = {ua, ub ? ub : ua, q};
+  CopyItem items[3];
+  int n = 0;
+  bool host = false;
+  for (int k = 0; k < 3; ++k) {
+    double* dst = c->edge + (size_t)k * c->nedge;
+    if (!src[k] || ctx_on_this_device(src[k], c->device)) {
+      items[n++] = {src[k], dst, eb};
+    } else {
+      CK(cudaMemcpyAsync(dst, src[k], eb, kind_from(src[k]), c->stream));
+      host = host || !on_device(src[k]);
+    }
+  }
+  CK(ctx_copy_list(items, n, c->stream));
   // host-sourced edge data must not be reused before the copies complete
-  if ((ua && !on_device(ua)) || (b && !on_device(b)) || (q && !on_device(q)))
-    CK(cudaStreamSynchronize(c->stream));
+  if (host) CK(cudaStreamSynchronize(c->stream));
   return LBM_OK;
 }
 
@@ -1215,25 +1214,31 @@ lbm_status lbm_save(lbm_ctx* c, void* buf, size_t bytes) {
   TRY(lbm_state_bytes(c, &need));
   if (!buf || bytes < need) return fail(LBM_ERR_ARG, "lbm_save: buffer smaller than lbm_state_bytes");
   const bool dev = on_device(buf);
-  const cudaMemcpyKind k = dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
   TRY(sync_mineral(c));
   BlobHeader h{kMagic, c->steps, c->p.nx, c->p.ny, c->p.precision, c->p.dissolution, c->nparts, 0};
-  if (dev) {
-    // the header travels as a kernel argument: nothing on this stack frame
-    // is read after the call returns, so a save into device memory need
-    // not wait
-    k_put_blob_header<<<1, 32, 0, c->stream>>>((unsigned char*)buf, h);
-    CK(cudaGetLastError());
-  } else {
-    memcpy(buf, &h, sizeof(h));
-  }
   Section s[16];
   const int n = state_sections(c, s);
   size_t off = align256(sizeof(BlobHeader));
+  if (ctx_on_this_device(buf, c->device)) {
+    // one launch; the header travels as a kernel argument: nothing on this
+    // stack frame is read after the call returns, so the save need not wait
+    CopyItem items[16];
+    for (int i = 0; i < n; ++i) {
+      items[i] = {s[i].ptr, (char*)buf + off, s[i].bytes};
+      off += align256(s[i].bytes);
+    }
+    CK(ctx_copy_list(items, n, c->stream, &h, buf, (int)sizeof(h)));
+    return LBM_OK;
+  }
+  // host memory, or memory that this device does not hold
+  const cudaMemcpyKind k = dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
+  if (dev) CK(cudaMemcpyAsync(buf, &h, sizeof(h), cudaMemcpyDefault, c->stream));
+  else memcpy(buf, &h, sizeof(h));
   for (int i = 0; i < n; ++i) {
     CK(cudaMemcpyAsync((char*)buf + off, s[i].ptr, s[i].bytes, k, c->stream));
     off += align256(s[i].bytes);
   }
+  if (dev) CK(cudaStreamSynchronize(c->stream));
   if (dev) return LBM_OK;
   return check_status(c);  // waits: the host blob is complete on return
 }
@@ -1256,18 +1261,29 @@ lbm_status lbm_restore(lbm_ctx* c, const void* buf, size_t bytes) {
   if (h.magic != kMagic || h.nx != c->p.nx || h.ny != c->p.ny ||
       h.precision != c->p.precision || h.dissolution != c->p.dissolution)
     return fail(LBM_ERR_STATE, "lbm_restore: blob does not belong to this lattice");
-  const cudaMemcpyKind k = dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
   Section s[16];
   const int n = state_sections(c, s);
   size_t off = align256(sizeof(BlobHeader));
-  for (int i = 0; i < n; ++i) {
-    CK(cudaMemcpyAsync(s[i].ptr, (const char*)buf + off, s[i].bytes, k, c->stream));
-    off += align256(s[i].bytes);
-  }
   // the blob holds no shares (every step writes those of its fluid nodes), and
   // a node that is solid again must not keep the one of its fluid life: a pass
   // reads a zero there while the node flips (lbm::flip_node)
-  if (c->p.dissolution) CK(cudaMemsetAsync(c->ureact, 0, (size_t)c->plane * 8, c->stream));
+  const size_t share_b = c->p.dissolution ? (size_t)c->plane * 8 : 0;
+  if (ctx_on_this_device(buf, c->device)) {
+    CopyItem items[17];
+    for (int i = 0; i < n; ++i) {
+      items[i] = {(const char*)buf + off, s[i].ptr, s[i].bytes};
+      off += align256(s[i].bytes);
+    }
+    items[n] = {nullptr, c->ureact, share_b};
+    CK(ctx_copy_list(items, n + 1, c->stream));
+  } else {
+    const cudaMemcpyKind k = dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
+    for (int i = 0; i < n; ++i) {
+      CK(cudaMemcpyAsync(s[i].ptr, (const char*)buf + off, s[i].bytes, k, c->stream));
+      off += align256(s[i].bytes);
+    }
+    if (share_b) CK(cudaMemsetAsync(c->ureact, 0, share_b, c->stream));
+  }
   c->steps = h.steps;
   c->nparts = h.nparts;
   if (!dev) CK(cudaStreamSynchronize(c->stream));

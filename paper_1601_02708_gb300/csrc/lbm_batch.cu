@@ -575,6 +575,9 @@ lbm_status lbm_batch_substeps(lbm_batch* b, int n, int eta, const double* const*
   if (!b) return fail(LBM_ERR_ARG, "null batch");
   if (n < 0 || eta < 1) return fail(LBM_ERR_ARG, "lbm_batch_substeps: need n >= 0, eta >= 1");
   if (n == 0) return LBM_OK;
+  // every member's edge data that the device holds in one launch (as 72 copies
+  // and clears those of 24 members took 440 us)
+  std::vector<CopyItem> items;
   for (size_t i = 0; i < b->m.size(); ++i) {
     lbm_ctx* c = b->m[i];
     const size_t eb = (size_t)c->nedge * sizeof(double);
@@ -582,10 +585,12 @@ lbm_status lbm_batch_substeps(lbm_batch* b, int n, int eta, const double* const*
                             u_dir_t1 ? u_dir_t1[i] : (u_dir_t0 ? u_dir_t0[i] : nullptr),
                             q_neu ? q_neu[i] : nullptr};
     for (int k = 0; k < 3; ++k) {
-      if (src[k]) BCK(cudaMemcpyAsync(c->edge + k * c->nedge, src[k], eb, cudaMemcpyDefault, b->stream));
-      else BCK(cudaMemsetAsync(c->edge + k * c->nedge, 0, eb, b->stream));
+      double* dst = c->edge + (size_t)k * c->nedge;
+      if (!src[k] || ctx_on_this_device(src[k], c->device)) items.push_back({src[k], dst, eb});
+      else BCK(cudaMemcpyAsync(dst, src[k], eb, cudaMemcpyDefault, b->stream));
     }
   }
+  BCK(ctx_copy_list(items.data(), (int)items.size(), b->stream));
   BCK(cudaStreamSynchronize(b->stream));  // host edge data may be reused after return
   return run_batch(b, n, eta);
 }

@@ -137,6 +137,20 @@ lbm_status ctx_make_map(const char* what, CUtensorMap* m, CUtensorMapDataType dt
 lbm_status ctx_check(const lbm_ctx* c);                    // null context
 lbm_status ctx_status(lbm_ctx* c);   // waits for the stream, reads the device error word
 bool ctx_on_device(const void* p);
+// Memory of this kind and device: what ctx_copy_list may read and write.
+bool ctx_on_this_device(const void* p, int device);
+// Copies within the device, one launch for up to kCopyMax of them (lbm_copy.cu);
+// a null source is zeros.  The regions do not overlap.  `head`, at most
+// kCopyHead bytes of host memory, is written to head_dst with the first launch
+// (it travels as a kernel argument).
+struct CopyItem {
+  const void* src;
+  void* dst;
+  size_t bytes;
+};
+constexpr int kCopyMax = 96, kCopyHead = 64;
+cudaError_t ctx_copy_list(const CopyItem* items, int n, cudaStream_t stream,
+                          const void* head = nullptr, void* head_dst = nullptr, int head_bytes = 0);
 // Copies the edge data of one call (NULL = zeros) into c->edge.
 lbm_status ctx_stage_edges(lbm_ctx* c, const double* ua, const double* ub, const double* q);
 // One step launch with explicit arguments (fin = c->f[c->cur] for the tile
