@@ -315,6 +315,14 @@ lbm_status sync_mineral(lbm_ctx* c) {
   return LBM_OK;
 }
 
+template <typename Real, int kWalls, int kRows>
+void launch_plain(lbm_ctx* c, const lbm::StepArgs<Real>& a, bool final_step) {
+  if (final_step)
+    lbm::lbm_step<Real, true, kWalls, kRows><<<c->sgrid, c->sblock, 0, c->stream>>>(a);
+  else
+    lbm::lbm_step<Real, false, kWalls, kRows><<<c->sgrid, c->sblock, 0, c->stream>>>(a);
+}
+
 // The step kernels are built without wall code and with the two precisions
 // of the maximum-entropy wall solve (walls_variant); a context runs the one
 // its wall mode needs.
@@ -331,10 +339,10 @@ lbm_status launch_step_kernels(lbm_ctx* c, const lbm::StepArgs<Real>& a, bool fi
           af, m, c->ntx, c->nty);
     if (final_step) c->nparts = c->tma_grid;
   } else {
-    if (final_step)
-      lbm::lbm_step<Real, true, kWalls><<<c->sgrid, c->sblock, 0, c->stream>>>(a);
+    if ((int)c->sblock.y == lbm::step_rows<Real>())
+      launch_plain<Real, kWalls, lbm::step_rows<Real>()>(c, a, final_step);
     else
-      lbm::lbm_step<Real, false, kWalls><<<c->sgrid, c->sblock, 0, c->stream>>>(a);
+      launch_plain<Real, kWalls, lbm::kSmallRows>(c, a, final_step);
     if (final_step) c->nparts = (int)(c->sgrid.x * c->sgrid.y);
   }
   CK(cudaGetLastError());
@@ -518,15 +526,17 @@ lbm_status init_impl(lbm_ctx* c, const uint8_t* solid, const double* vel,
   c->nedge = 2 * (p.nx + p.ny);
   c->block = dim3(lbm::kBX, lbm::kBY);
   c->grid = dim3((p.nx + lbm::kBX - 1) / lbm::kBX, (p.ny + lbm::kBY - 1) / lbm::kBY);
-  {
-    const int rows = p.precision == 64 ? lbm::step_rows<double>() : lbm::step_rows<float>();
-    c->sblock = dim3(lbm::kBX, rows);
-    c->sgrid = dim3((p.nx + lbm::kBX - 1) / lbm::kBX, (p.ny + rows - 1) / rows);
-  }
   const size_t plane_b = (size_t)c->plane * c->esize;
   const int per_x = p.edge[0] == LBM_EDGE_PERIODIC;
   CK(cudaGetDevice(&c->device));
   CK(cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, c->device));
+  {
+    const bool f64 = p.precision == 64;
+    const bool few = f64 && (long long)c->grid.x * c->grid.y < 2LL * c->num_sms;  // 32 x 8 blocks
+    const int rows = few ? lbm::kSmallRows : f64 ? lbm::step_rows<double>() : lbm::step_rows<float>();
+    c->sblock = dim3(lbm::kBX, rows);
+    c->sgrid = dim3((p.nx + lbm::kBX - 1) / lbm::kBX, (p.ny + rows - 1) / rows);
+  }
   {
     const long long blocks = ((long long)p.nx * p.ny + lbm::kDThreads - 1) / lbm::kDThreads;
     const long long cap = 8LL * c->num_sms;  // 8 resident blocks of 256 per SM

@@ -48,6 +48,11 @@ template <typename Real>
 __host__ __device__ constexpr int step_rows() {
   return sizeof(Real) == 4 ? 2 : 8;
 }
+// FP64 lattices of fewer than two 32 x 8 blocks per SM run 32 x 2: there the
+// step is as long as the SM with the most warps keeps its FP64 pipe, and small
+// blocks spread (a 256 x 64 lattice: 4 warps on every SM, not 8 on 64 of 152):
+// 8.1 -> 5.7 us a substep there, 13.0 -> 10.5 at 331 x 203 with pores.
+constexpr int kSmallRows = 2;
 
 template <typename Real>
 struct StepArgs {
@@ -450,13 +455,13 @@ __device__ __forceinline__ PreSrc<Real> preload(const StepArgs<Real>& a, long lo
 
 // Generic step: one thread per node, inputs from global memory.  The FP64
 // lattice's step, and the FP32 one on large lattices (lbm_set_kernel).
-template <typename Real, bool kFinal, int kWalls = 0>
+template <typename Real, bool kFinal, int kWalls = 0, int kBY = step_rows<Real>()>
 // FP32: 24 blocks of 64 per SM (40 registers, as many threads as six blocks
 // of 256) keep more loads in flight than fewer threads; FP64 keeps four
-// blocks of 256 (64 registers) for its arithmetic.
-__global__ void __launch_bounds__(kBX * step_rows<Real>(), sizeof(Real) == 4 ? 24 : 4)
+// blocks of 256, or as many threads in blocks of 64 (64 registers), for its
+// arithmetic.
+__global__ void __launch_bounds__(kBX * kBY, sizeof(Real) == 4 ? 24 : 32 / kBY)
     lbm_step(const StepArgs<Real> a) {
-  constexpr int kBY = step_rows<Real>();
   __shared__ double red[kBX * kBY / 32];
   if (a.dissolve_state && blockIdx.x + blockIdx.y + threadIdx.x + threadIdx.y == 0)
     open_pass(a.dissolve_state);
