@@ -532,7 +532,7 @@ lbm_status init_impl(lbm_ctx* c, const uint8_t* solid, const double* vel,
   CK(cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, c->device));
   {
     const bool f64 = p.precision == 64;
-    const bool few = f64 && (long long)c->grid.x * c->grid.y < 2LL * c->num_sms;  // 32 x 8 blocks
+    const bool few = f64 && (long long)c->grid.x * c->grid.y < 5LL * c->num_sms;  // 32 x 8 blocks
     const int rows = few ? lbm::kSmallRows : f64 ? lbm::step_rows<double>() : lbm::step_rows<float>();
     c->sblock = dim3(lbm::kBX, rows);
     c->sgrid = dim3((p.nx + lbm::kBX - 1) / lbm::kBX, (p.ny + rows - 1) / rows);

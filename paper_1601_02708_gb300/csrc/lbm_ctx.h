@@ -204,6 +204,9 @@ inline lbm::StepArgs<Real> step_args(lbm_ctx* c, double frac) {
   a.react_mode = c->p.react_mode;
   a.dissolution = c->p.dissolution;
   a.omega = (Real)(1.0 / c->p.tau);
+  a.om1 = (Real)1 - a.omega;
+  a.om_half = a.omega / 2;
+  a.om_third = a.omega / 3;
   a.k_scalar = (Real)c->p.k_scalar;
   a.frac = frac;
   return a;

@@ -48,10 +48,11 @@ template <typename Real>
 __host__ __device__ constexpr int step_rows() {
   return sizeof(Real) == 4 ? 2 : 8;
 }
-// FP64 lattices of fewer than two 32 x 8 blocks per SM run 32 x 2: there the
+// FP64 lattices of fewer than five 32 x 8 blocks per SM run 32 x 2: there the
 // step is as long as the SM with the most warps keeps its FP64 pipe, and small
 // blocks spread (a 256 x 64 lattice: 4 warps on every SM, not 8 on 64 of 152):
-// 8.1 -> 5.7 us a substep there, 13.0 -> 10.5 at 331 x 203 with pores.
+// 8.1 -> 5.7 us a substep there, 13.0 -> 10.5 at 331 x 203 with pores, 21.2 ->
+// 18.1 at 512 x 256, whose 512 blocks of 32 x 8 are three or four to an SM.
 constexpr int kSmallRows = 2;
 
 template <typename Real>
@@ -93,6 +94,7 @@ struct StepArgs {
   int react_mode;
   int dissolution;
   Real omega;  // 1 / tau
+  Real om1, om_half, om_third;  // 1 - omega, omega / 2, omega / 3
   Real k_scalar;
   double frac;  // j / eta of this substep
 };
@@ -172,29 +174,36 @@ __device__ __forceinline__ void equilibrium(Real (&feq)[9], Real u, Real vx, Rea
 // summing to the post-reaction mass in FP32.
 template <typename Real>
 __device__ __forceinline__ void collide(Real (&f)[9], Real u, Real vx, Real vy,
-                                        Real omega, Real kr) {
-  const Real base = (Real)1 - (Real)1.5 * (vx * vx + vy * vy);
+                                        const StepArgs<Real>& a, Real kr) {
+  const Real omega = a.omega;
   if constexpr (sizeof(Real) == 8) {
     // FP64: the FP64 pipe bounds the step, so the form with the fewest FP64
-    // operations (43 instead of 59, and 8 for u): the rest population in closed
-    // form (the weights sum to one to 1e-17), w u per weight instead of per
-    // pair, and each population two fused multiply-adds.  A ten-step call
-    // at 1024 x 1024 went from 1242 to 1180 us.
-    const Real om1 = (Real)1 - omega, c45 = (Real)4.5 * omega, c3 = (Real)3 * omega;
-    const Real sym0 = omega * base - kr;
-    f[0] = om1 * f[0] + ((Real)w_of(0) * u) * sym0;
-    const Real wu1 = (Real)w_of(1) * u, wu5 = (Real)w_of(5) * u;
-    const Real ev[4] = {vx, vy, vx + vy, vy - vx};
+    // operations, 38 a node and 8 for u: the rest population in closed form
+    // (the weights sum to one to 1e-17), the weights taken into factors that
+    // the host forms (4.5 w = 1/2 and 1/8, 3 w = 1/3 and 1/12), each
+    // population two fused multiply-adds.  A ten-step call at 1024 x 1024 went
+    // from 1072 to 926 us by this form (43 operations before) and by shares
+    // without a division (kPerW).
+    const Real x2 = vx * vx, y2 = vy * vy;
+    const Real base = (Real)1 - (Real)1.5 * (x2 + y2);
+    const Real us = u * (omega * base - kr);
+    const Real a1 = a.om_half * u, a5 = (Real)0.25 * a1;
+    const Real b1 = a.om_third * u, b5 = (Real)0.25 * b1;
+    const Real s1 = (Real)w_of(1) * us, s5 = (Real)w_of(5) * us;
+    const Real ne = vx + vy, nw = vy - vx;
+    f[0] = a.om1 * f[0] + (Real)w_of(0) * us;
+    const Real t[4] = {a1 * x2 + s1, a1 * y2 + s1, a5 * (ne * ne) + s5, a5 * (nw * nw) + s5};
+    const Real ev[4] = {vx, vy, ne, nw};
 #pragma unroll
     for (int p = 0; p < 4; ++p) {
       const int i = p < 2 ? p + 1 : p + 3, o = opp_of(i);
-      const Real wu = p < 2 ? wu1 : wu5;
-      const Real sym = wu * (c45 * (ev[p] * ev[p]) + sym0), e = c3 * ev[p];
-      f[i] = wu * e + (om1 * f[i] + sym);
-      f[o] = (om1 * f[o] + sym) - wu * e;
+      const Real b = p < 2 ? b1 : b5;
+      f[i] = b * ev[p] + (a.om1 * f[i] + t[p]);
+      f[o] = (a.om1 * f[o] + t[p]) - b * ev[p];
     }
     return;
   }
+  const Real base = (Real)1 - (Real)1.5 * (vx * vx + vy * vy);
   const Real om1 = (Real)1 - omega;
   // the factors that do not depend on the direction, formed once
   const Real sym0 = omega * base - kr;
@@ -254,6 +263,18 @@ struct GlobalSrc {
   __device__ __forceinline__ Real kf() const { return a.kf[nd()]; }
 };
 
+// 1 / W_s by c = 36 W_s = 1 .. 20, and 0 for c = 0: a division in the FP64 step
+// is a dozen operations of its pipe, in nearly every warp of a pore lattice.
+struct PerW {
+  double v[21];
+};
+constexpr PerW make_per_w() {
+  PerW t{};
+  for (int c = 1; c < 21; ++c) t.v[c] = 36.0 / c;
+  return t;
+}
+__device__ const PerW kPerW = make_per_w();
+
 // Reaction share of a near-solid node, stored for the dissolution pass:
 // r = k u / W_s on the FP64 lattice; the concentration and 36 W_s on the FP32
 // lattice (the pass forms r in FP64).  `post` holds the node's links to solid
@@ -263,8 +284,8 @@ __device__ __forceinline__ void store_share(const StepArgs<Real>& a, long long n
                                             Real u, uint32_t post, bool ghosts, int x, int y) {
   const int na = __popc(post & 0x0Fu), nd = __popc(post & 0xF0u);
   if constexpr (sizeof(Real) == 8) {
-    const double wsolid = (double)na * w_of(1) + (double)nd * w_of(5);
-    store_node((double*)a.ureact, n, post ? (double)kr * (double)u / wsolid : 0.0, ghosts, x, y,
+    // (kPerW[0] = 0)
+    store_node((double*)a.ureact, n, ((double)kr * (double)u) * kPerW.v[4 * na + nd], ghosts, x, y,
                a.nx, a.ny, a.pitch, a.per_x, a.per_y, a.plane, a.status);
   } else {
     ShareF32 v;
@@ -369,8 +390,12 @@ __device__ __forceinline__ double step_node(const StepArgs<Real>& a, const Src& 
     }
   }
   Real u = f[0];
+  if constexpr (sizeof(Real) == 8) {  // a tree: an FP64 operation is slow to return
+    u = (((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7]))) + f[8];
+  } else {
 #pragma unroll
-  for (int i = 1; i < 9; ++i) u += f[i];
+    for (int i = 1; i < 9; ++i) u += f[i];
+  }
   // the first moment through the east column (outlet flux of lbm_diagnostics)
   if (kEdge && x == a.nx - 1 && a.jflux && !own_solid)
     a.jflux[y] = ((double)f[1] + (double)f[5] + (double)f[8]) -
@@ -382,7 +407,7 @@ __device__ __forceinline__ double step_node(const StepArgs<Real>& a, const Src& 
   Real kr = (Real)0;
   if (a.react_mode == kReactBulk || (a.react_mode == kReactSurface && near_solid))
     kr = a.kf ? src.kf() : a.k_scalar;
-  collide(f, u, src.vx(), src.vy(), a.omega, kr);
+  collide(f, u, src.vx(), src.vy(), a, kr);
   if (kLight && own_solid) {  // a solid lane: zeros (pending), or nothing to keep
 #pragma unroll
     for (int i = 0; i < 9; ++i) f[i] = (Real)0;
@@ -559,7 +584,7 @@ __global__ void __launch_bounds__(kBX * kBY)
       Real kr = (Real)0;
       if (a.react_mode == kReactBulk || (a.react_mode == kReactSurface && near_solid))
         kr = a.kf ? a.kf[n] : a.k_scalar;
-      collide(f, u, vx, vy, a.omega, kr);
+      collide(f, u, vx, vy, a, kr);
 #pragma unroll
       for (int i = 0; i < 9; ++i)
         store_node(a.fout + i * a.plane, n, f[i], ghosts, x, y, a.nx, a.ny, a.pitch,
