@@ -88,21 +88,34 @@ __device__ __forceinline__ void adjoint_node(const AdjArgs<Real>& a, int x, int 
   using namespace lbm;
   const long long nn = dbg_idx(n, a.plane, a.status, kSiteAdjNode);
   const long long lim = 9 * a.plane;
+  // every load in one round, the gathers as if no neighbour were solid; nodes
+  // with solid neighbours (and sides) then put theirs right
   const uint32_t w = a.link[nn];
-  if (w & kOwnSolid) return;
   Real lam[9];
   lam[0] = a.mu_in[nn];
 #pragma unroll
-  for (int j = 1; j < 9; ++j) {
-    const int jb = opp_of(j);
-    if (kEdge && (w & up_bit(kUpOutShift, jb))) {
-      lam[j] = (Real)0;
-    } else if (w & up_bit(kUpSolidShift, jb)) {
-      lam[j] = a.mu_in[dbg_idx(jb * a.plane + n, lim, a.status, kSiteAdjGather)];
-    } else {
-      lam[j] = a.mu_in[dbg_idx(j * a.plane + n + cx_of(j) + (long long)cy_of(j) * a.pitch, lim,
-                               a.status, kSiteAdjGather)];
-    }
+  for (int j = 1; j < 9; ++j)
+    lam[j] = a.mu_in[dbg_idx(j * a.plane + n + cx_of(j) + (long long)cy_of(j) * a.pitch, lim,
+                             a.status, kSiteAdjGather)];
+  const Real vx = a.vel[nn], vy = a.vel[a.plane + nn];
+  Real kn = a.k_scalar, un = (Real)0;
+  float g32 = 0.f;
+  if (a.react_mode != kReactNone) {
+    if (a.kf) kn = a.kf[nn];
+    un = a.u_n[nn];
+    if constexpr (sizeof(Real) == 4) g32 = a.gk32[nn];
+  }
+  if (w & kOwnSolid) return;
+  if (w & 0xFFu) {
+#pragma unroll
+    for (int j = 1; j < 9; ++j)
+      if (w & up_bit(kUpSolidShift, opp_of(j)))
+        lam[j] = a.mu_in[dbg_idx(opp_of(j) * a.plane + n, lim, a.status, kSiteAdjGather)];
+  }
+  if (kEdge) {
+#pragma unroll
+    for (int j = 1; j < 9; ++j)
+      if (w & up_bit(kUpOutShift, opp_of(j))) lam[j] = (Real)0;
   }
   const uint32_t post = (w >> kUpPostShift) & 0xFFu;
   const bool reactive =
@@ -111,12 +124,11 @@ __device__ __forceinline__ void adjoint_node(const AdjArgs<Real>& a, int x, int 
 #pragma unroll
   for (int i = 1; i < 9; ++i) wl += (Real)w_of(i) * lam[i];
   if (reactive) {
-    if constexpr (sizeof(Real) == 4) a.gk32[nn] -= a.u_n[nn] * wl;
-    else a.gk[nn] -= (double)a.u_n[nn] * (double)wl;
+    if constexpr (sizeof(Real) == 4) a.gk32[nn] = g32 - un * wl;
+    else a.gk[nn] -= (double)un * (double)wl;
   }
   if (kInit) return;
-  const Real kr = reactive ? (a.kf ? a.kf[nn] : a.k_scalar) : (Real)0;
-  const Real vx = a.vel[nn], vy = a.vel[a.plane + nn];
+  const Real kr = reactive ? kn : (Real)0;
   const Real base = (Real)1 - (Real)1.5 * (vx * vx + vy * vy);
   // sum_i w_i P_i lambda_i, by opposite pairs (P differs in the sign of 3 e.v)
   Real wp = (Real)w_of(0) * base * lam[0];
@@ -219,10 +231,13 @@ __device__ __forceinline__ void adjoint_node(const AdjArgs<Real>& a, int x, int 
 
 // One adjoint step (kInit: the gather of lambda^0 and the first collision's
 // rate term only).  One thread per node in blocks of one warp (32 x
-// kAdjRows): the reverse step is bound by the latency of its gathers, and
+// kAdjRows): the reverse step is bound by the latency of its loads, and
 // one-warp blocks leave no slot waiting for a block's slowest warp.  One
 // 5000-step call at 512^2 took 113, 101, 89 and 84 ms with 8, 4, 2 and 1
-// rows per block.
+// rows per block (with the boundary mixing in FP64; without it 2 rows are
+// as good and 4 are 6% slower).  One gradient over 500 steps there: 7.67 ms
+// with each gather waiting for the link word, 7.33 with every load in one round
+// (56 registers; held to 48 it spills: 7.62).
 constexpr int kAdjRows = 1;
 template <typename Real, bool kInit>
 __global__ void __launch_bounds__(lbm::kBX * kAdjRows) lbm_adjoint_step(const AdjArgs<Real> a) {
