@@ -199,19 +199,25 @@ class LBM:
         ua / ub [n_edge] = dJ/d(Dirichlet data at the start / end),
         q [n_edge] = dJ/d(Neumann data), side [4] = dJ/d(one Dirichlet
         value held on the whole W, E, S, N side)).  Fixed mask only."""
+        gk = np.empty((self.ny, self.nx))
+        ga, gb, gq = (np.empty(self.n_edge) for _ in range(3))
+        J, gs = self._adjoint(n, eta, u_dir_t0, u_dir_t1, q_neu, stride, gk.ctypes.data,
+                              ga.ctypes.data, gb.ctypes.data, gq.ctypes.data)
+        return dict(J=J, k=gk, ua=ga, ub=gb, q=gq, side=gs)
+
+    def _adjoint(self, n, eta, u_dir_t0, u_dir_t1, q_neu, stride, gk, ga=None, gb=None, gq=None):
+        """lbm_adjoint into addresses (host or device, None to leave one out);
+        returns J and the side gradients.  Waits for the results."""
         keep = []
         m = self.n_edge
         a = _in_ptr(u_dir_t0, "f64", m, keep)
         b = _in_ptr(u_dir_t1, "f64", m, keep)
         q = _in_ptr(q_neu, "f64", m, keep)
         J = ctypes.c_double()
-        gk = np.empty((self.ny, self.nx))
-        ga, gb, gq = (np.empty(m) for _ in range(3))
         gs = np.empty(4)
         check(self._lib.lbm_adjoint(self.handle, int(n), int(eta), int(stride), a, b, q,
-                                    ctypes.byref(J), gk.ctypes.data, ga.ctypes.data,
-                                    gb.ctypes.data, gq.ctypes.data, gs.ctypes.data))
-        return dict(J=J.value, k=gk, ua=ga, ub=gb, q=gq, side=gs)
+                                    ctypes.byref(J), gk, ga, gb, gq, gs.ctypes.data))
+        return J.value, gs
 
     KERNELS = {"auto": 0, "generic": 1, "tma": 2}
 
@@ -406,14 +412,19 @@ def _breakthrough_class():
             ud = np.zeros(lbm.n_edge)
             if lbm.edges[0] == DIRICHLET:
                 ud[:lbm.ny] = cin
-            r = lbm.adjoint(n, 1, ud, ud, None, stride)
             dev = k_field.device if torch.is_tensor(k_field) else "cpu"
-            gk = torch.as_tensor(r["k"], device=dev).to(k_field.dtype).reshape(k_field.shape)
-            gc = float(r["side"][0])  # dJ/dc_in of the west side, from the library
+            # dJ/dk stays where the rate field is, and the edge gradients are left
+            # out: 4.25 -> 4.16 ms for 225 checkpointed steps at 331 x 203
+            gk = torch.empty(lbm.ny, lbm.nx, dtype=torch.float64, device=dev)
+            if gk.is_cuda:  # the library's stream may reuse memory that torch's still reads
+                torch.cuda.current_stream(gk.device).synchronize()
+            J, side = lbm._adjoint(n, 1, ud, ud, None, stride, gk.data_ptr())
+            gk = gk.to(k_field.dtype).reshape(k_field.shape)
+            gc = float(side[0])  # dJ/dc_in of the west side, from the library
             ctx.save_for_backward(gk)
             ctx.gc = gc
             ctx.cin_like = c_in if torch.is_tensor(c_in) else None
-            return torch.tensor(r["J"], dtype=torch.float64, device=dev)
+            return torch.tensor(J, dtype=torch.float64, device=dev)
 
         @staticmethod
         def backward(ctx, gJ):
