@@ -96,8 +96,8 @@ enum { LBM_SIDE_W = 0, LBM_SIDE_E = 1, LBM_SIDE_S = 2, LBM_SIDE_N = 3 };
 typedef struct {
   int nx, ny;        /* lattice nodes, each >= 2; ny <= 65535 (a launch's
                         block index in y numbers the rows) */
-  int precision;     /* 32: FP32 populations and arithmetic (FP64 boundary
-                        solves, reaction shares, mineral and sums); 64: FP64
+  int precision;     /* 32: FP32 populations and arithmetic (boundary
+                        solves in double-float, mineral and sums in FP64); 64: FP64
                         throughout */
   int edge[4];       /* lbm_edge_kind of the W, E, S, N sides */
   double tau;        /* BGK relaxation time (Eq. "Collision"), > 1/2 */

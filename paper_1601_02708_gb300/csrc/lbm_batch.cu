@@ -85,7 +85,7 @@ __device__ __forceinline__ void tensormap_acquire(const CUtensorMap* m) {
 // each tile's mass partial is summed in a fixed order by consumer warp 0
 // once the other warps have posted theirs (an mbarrier per stage).  The
 // boundary warp steps the nodes on every member's non-periodic sides from
-// global memory (FP64 solves), in chunks of 32 nodes of one member:
+// global memory (maximum-entropy solves), in chunks of 32 nodes of one member:
 // otask[32 c + lane] = (member, padded node index or -1, partial slot, 0).
 template <bool kFinal, int kWalls = 0>
 __global__ void __launch_bounds__(lbm::kTmaBlock, 1)
@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(lbm::kTmaBlock, 1)
       }
     }
   } else if (warp == kBoundaryWarp) {
-    // ---- boundary nodes of every member: FP64 solves beside the pipeline --
+    // ---- boundary nodes of every member: solves beside the pipeline -------
     for (int ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
       const int4 task = otask[32 * ch + lane];
       const StepArgs<float>& a = args[task.x].a;  // one member per chunk

@@ -29,7 +29,7 @@ constexpr int kBatchPlainShapes = 6;
 
 // One tile list over every member: tile (member, x0, y0, index | rate bit).
 // Each block walks tiles t, t + grid, ...; the nodes of a tile step in place
-// (boundary solves inline, in FP64).
+// (boundary solves inline).
 template <typename Real, bool kFinal, int kBY, int kR, int kWalls>
 __global__ void __launch_bounds__(32 * kBY)
     lbm_step_batch(const ArgSlot<Real>* __restrict__ args, const int4* __restrict__ tiles,

@@ -366,8 +366,8 @@ __device__ __forceinline__ double step_node(const StepArgs<Real>& a, const Src& 
     const unsigned unknown = ((w >> kUpOutShift) & 0xFFu) << 1;  // bit i: direction i
     if (unknown) {
       // Boundary node: Dirichlet wins at corners, else Neumann.  The solves
-      // run in FP64 from the FP64 edge data on either lattice; only their
-      // results are rounded to the lattice's precision.
+      // carry the FP64 edge data on either lattice (double-float on the FP32
+      // one); only their results are rounded to the lattice's precision.
       int dside, nside, sx, sy;
       edge_kind(a.edge, x, y, a.nx, a.ny, &dside, &nside, &sx, &sy);
       bool bad;

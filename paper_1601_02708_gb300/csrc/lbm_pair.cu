@@ -8,7 +8,7 @@
 // the producer brings both fields' population boxes (with their one-node
 // halo) but the velocity and link-word boxes once; 12 consumer warps update
 // each field's 384 nodes; the boundary warp steps both fields' nodes on the
-// Dirichlet/Neumann sides (FP64 solves).  Four rows instead of eight keep
+// Dirichlet/Neumann sides (maximum-entropy solves).  Four rows instead of eight keep
 // four pipeline stages of both fields in shared memory.  Each field computes
 // exactly what stepping its lattice alone computes.
 #include <cuda.h>

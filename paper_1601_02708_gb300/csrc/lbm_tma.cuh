@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(kTmaBlock, 1)
       }
     }
   } else if (warp == kBoundaryWarp) {
-    // ---- boundary nodes: FP64 maximum-entropy solves beside the pipeline --
+    // ---- boundary nodes: maximum-entropy solves beside the pipeline -------
     // (every lane runs the same trip count; lanes past the list idle)
     for (int e0 = blockIdx.x * 32; e0 < a.n_open; e0 += gridDim.x * 32) {
       const int e = e0 + lane;
