@@ -120,27 +120,33 @@ __device__ __forceinline__ void adjoint_node(const AdjArgs<Real>& a, int x, int 
   const uint32_t post = (w >> kUpPostShift) & 0xFFu;
   const bool reactive =
       a.react_mode == kReactBulk || (a.react_mode == kReactSurface && post != 0u);
-  Real wl = (Real)w_of(0) * lam[0];
-#pragma unroll
-  for (int i = 1; i < 9; ++i) wl += (Real)w_of(i) * lam[i];
+  // sum_i w_i lambda_i about lambda_0: the weights sum to one in exact
+  // arithmetic, rounded to FP32 to 1 + 7.5e-9, which would grow the gradient by
+  // as much with every step
+  const Real la = ((lam[1] - lam[0]) + (lam[3] - lam[0])) + ((lam[2] - lam[0]) + (lam[4] - lam[0]));
+  const Real ld = ((lam[5] - lam[0]) + (lam[7] - lam[0])) + ((lam[6] - lam[0]) + (lam[8] - lam[0]));
+  const Real wl = lam[0] + ((Real)w_of(1) * la + (Real)w_of(5) * ld);
   if (reactive) {
     if constexpr (sizeof(Real) == 4) a.gk32[nn] = g32 - un * wl;
     else a.gk[nn] -= (double)un * (double)wl;
   }
   if (kInit) return;
   const Real kr = reactive ? kn : (Real)0;
-  const Real base = (Real)1 - (Real)1.5 * (vx * vx + vy * vy);
-  // sum_i w_i P_i lambda_i, by opposite pairs (P differs in the sign of 3 e.v)
-  Real wp = (Real)w_of(0) * base * lam[0];
+  const Real vv = (Real)1.5 * (vx * vx + vy * vy);
+  // sum_i w_i P_i lambda_i, the part of P that depends on v by opposite pairs
+  // (which differ in the sign of 3 e.v) and about lambda_0: that part's weighted
+  // sum is zero
+  Real wv = (Real)0;
 #pragma unroll
   for (int p = 0; p < 4; ++p) {
     const int i = p < 2 ? p + 1 : p + 3;
     const int o = opp_of(i);
     const Real ev = (Real)cx_of(i) * vx + (Real)cy_of(i) * vy;
-    const Real sym = base + (Real)4.5 * ev * ev;
-    const Real anti = (Real)3 * ev;
-    wp += (Real)w_of(i) * ((sym + anti) * lam[i] + (sym - anti) * lam[o]);
+    const Real sym = (Real)4.5 * ev * ev - vv;
+    wv += (Real)w_of(i) * (sym * ((lam[i] - lam[0]) + (lam[o] - lam[0])) +
+                           (Real)3 * ev * (lam[i] - lam[o]));
   }
+  const Real wp = wl + wv;
   Real s = a.omega * wp - kr * wl;
   if (kEdge && x == a.nx - 1) s += (Real)1;  // u^n counts in J
   const Real om1 = (Real)1 - a.omega;
