@@ -157,6 +157,22 @@ __global__ void k_count_solid(const uint32_t* __restrict__ link, int nx, int ny,
   if ((threadIdx.x & 31) == 0 && c) atomicAdd(out, c);
 }
 
+// Zero reaction shares at the solid nodes (and their ghost images; the ghost
+// rows beyond a slab's shared sides hold the neighbour's, which the halo brings).
+__global__ void k_clear_solid_shares(const uint32_t* __restrict__ link,
+                                     unsigned long long* __restrict__ share, int nx, int ny,
+                                     int pitch, int per_x, int per_y, long long plane,
+                                     int* status) {
+  const long long total = (long long)nx * ny;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
+       i += (long long)gridDim.x * blockDim.x) {
+    const int y = (int)(i / nx), x = (int)(i - (long long)y * nx);
+    const long long n = (long long)(y + kYO) * pitch + (x + kXO);
+    if (link[n] & lbm::kOwnSolid)
+      lbm::store_node(share, n, 0ull, true, x, y, nx, ny, pitch, per_x, per_y, plane, status);
+  }
+}
+
 // Fixed-order FP64 reductions for lbm_diagnostics (one block).
 __global__ void k_diag(const double* __restrict__ partial, int nparts,
                        const double* __restrict__ jnode, const double* __restrict__ jflux,
@@ -1274,25 +1290,30 @@ lbm_status lbm_restore(lbm_ctx* c, const void* buf, size_t bytes) {
   Section s[16];
   const int n = state_sections(c, s);
   size_t off = align256(sizeof(BlobHeader));
-  // the blob holds no shares (every step writes those of its fluid nodes), and
-  // a node that is solid again must not keep the one of its fluid life: a pass
-  // reads a zero there while the node flips (lbm::flip_node)
-  const size_t share_b = c->p.dissolution ? (size_t)c->plane * 8 : 0;
   if (ctx_on_this_device(buf, c->device)) {
-    CopyItem items[17];
+    CopyItem items[16];
     for (int i = 0; i < n; ++i) {
       items[i] = {(const char*)buf + off, s[i].ptr, s[i].bytes};
       off += align256(s[i].bytes);
     }
-    items[n] = {nullptr, c->ureact, share_b};
-    CK(ctx_copy_list(items, n + 1, c->stream));
+    CK(ctx_copy_list(items, n, c->stream));
   } else {
     const cudaMemcpyKind k = dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     for (int i = 0; i < n; ++i) {
       CK(cudaMemcpyAsync(s[i].ptr, (const char*)buf + off, s[i].bytes, k, c->stream));
       off += align256(s[i].bytes);
     }
-    if (share_b) CK(cudaMemsetAsync(c->ureact, 0, share_b, c->stream));
+  }
+  if (c->p.dissolution) {
+    // the blob holds no shares.  Those of fluid nodes stay: every step writes
+    // them anew, and where a pass is due (a slab's first one, or between
+    // lbm_step_stream and lbm_step_dissolve) it reads the ones that are there.
+    // A node that is solid again must not keep the one of its fluid life: a
+    // pass reads a zero there while the node flips (lbm::flip_node)
+    k_clear_solid_shares<<<c->dgrid, lbm::kDThreads, 0, c->stream>>>(
+        c->link, (unsigned long long*)c->ureact, c->p.nx, c->p.ny, c->pitch,
+        c->p.edge[0] == LBM_EDGE_PERIODIC, c->p.edge[2] == LBM_EDGE_PERIODIC, c->plane, c->status);
+    CK(cudaGetLastError());
   }
   c->steps = h.steps;
   c->nparts = h.nparts;
