@@ -81,6 +81,20 @@ __global__ void k_pitch_in(const double* __restrict__ src, T* __restrict__ dst, 
   }
 }
 
+// The rate field, with its ghost images across periodic sides: the FP32
+// lattice's dissolution pass reads k beside the share of a node across them.
+template <typename T>
+__global__ void k_rate_in(const double* __restrict__ src, T* __restrict__ dst, int nx, int ny,
+                          int pitch, int per_x, int per_y) {
+  const long long total = (long long)nx * ny;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
+       i += (long long)gridDim.x * blockDim.x) {
+    const int y = (int)(i / nx), x = (int)(i - (long long)y * nx);
+    lbm::store_node(dst, (long long)(y + kYO) * pitch + (x + kXO), (T)src[i], true, x, y, nx, ny,
+                    pitch, per_x, per_y);
+  }
+}
+
 // Link word of every interior node (see lbm_lattice.cuh) from the caller's
 // solid array of the whole lattice ([nyg][nx]); the context holds rows
 // y0 .. y0 + nyl - 1 of it (all of it unless the lattice is split into
@@ -435,6 +449,16 @@ lbm_status stage_doubles(lbm_ctx* c, const double* src, size_t count, double** o
   return LBM_OK;
 }
 
+// The rate field of the lattice from a device array [ny][nx].
+void put_rate(lbm_ctx* c, const double* dk) {
+  const int nx = c->p.nx, ny = c->p.ny, g = grid1d((long long)nx * ny);
+  const int per_x = c->p.edge[0] == LBM_EDGE_PERIODIC, per_y = c->p.edge[2] == LBM_EDGE_PERIODIC;
+  if (c->esize == 8)
+    k_rate_in<double><<<g, 256, 0, c->stream>>>(dk, (double*)c->kf, nx, ny, c->pitch, per_x, per_y);
+  else
+    k_rate_in<float><<<g, 256, 0, c->stream>>>(dk, (float*)c->kf, nx, ny, c->pitch, per_x, per_y);
+}
+
 void free_ctx(lbm_ctx* c) {
   if (!c) return;
   for (auto& kv : c->graphs) cudaGraphExecDestroy(kv.second.exec);
@@ -682,11 +706,10 @@ lbm_status init_impl(lbm_ctx* c, const uint8_t* solid, const double* vel,
   }
   if (c->esize == 8) {
     k_pitch_in<double><<<g, 256, 0, c->stream>>>(dvel, (double*)c->vel, p.nx, p.ny, c->pitch, 2, 0.0);
-    if (dk) k_pitch_in<double><<<g, 256, 0, c->stream>>>(dk, (double*)c->kf, p.nx, p.ny, c->pitch, 1, 0.0);
   } else {
     k_pitch_in<float><<<g, 256, 0, c->stream>>>(dvel, (float*)c->vel, p.nx, p.ny, c->pitch, 2, 0.0);
-    if (dk) k_pitch_in<float><<<g, 256, 0, c->stream>>>(dk, (float*)c->kf, p.nx, p.ny, c->pitch, 1, 0.0);
   }
+  if (dk) put_rate(c, dk);
   if (p.dissolution)
     k_pitch_in<double><<<g, 256, 0, c->stream>>>(dmin, c->mineral, p.nx, p.ny, c->pitch, 1, 1.0);
   k_count_solid<<<grid1d((long long)nxy), 256, 0, c->stream>>>(
@@ -1079,11 +1102,7 @@ lbm_status lbm_set_rate_field(lbm_ctx* c, const double* k_field) {
   double* dk = nullptr;
   bool owned = false;
   TRY(stage_doubles(c, k_field, nxy, &dk, &owned));
-  const int g = grid1d((long long)nxy);
-  if (c->esize == 8)
-    k_pitch_in<double><<<g, 256, 0, c->stream>>>(dk, (double*)c->kf, c->p.nx, c->p.ny, c->pitch, 1, 0.0);
-  else
-    k_pitch_in<float><<<g, 256, 0, c->stream>>>(dk, (float*)c->kf, c->p.nx, c->p.ny, c->pitch, 1, 0.0);
+  put_rate(c, dk);
   const cudaError_t e = cudaGetLastError();
   if (owned) {
     cudaStreamSynchronize(c->stream);

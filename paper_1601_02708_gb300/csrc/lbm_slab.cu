@@ -10,7 +10,8 @@
 //   phase 0, after the fused step: the three populations that stream across
 //     the cut (S side: directions 4, 7, 8 leave downwards; N side: 2, 5, 6)
 //     and, with dissolution, the reaction shares of the boundary row, which
-//     the neighbour's dissolution pass gathers;
+//     the neighbour's dissolution pass gathers, on the FP32 lattice with its
+//     rates where it has a rate field (the pass multiplies them there);
 //   phase 1, after the dissolution pass: the link words of the boundary row,
 //     whose own bits (solid, turning fluid) decide the links that cross the
 //     cut: the receiver sets them from the ghost row (a link "solid while
@@ -47,15 +48,17 @@ __host__ __device__ inline int plane_of(int side, int k) {
 
 template <typename Real>
 __global__ void k_pack0(const Real* __restrict__ f, const void* __restrict__ share,
-                        int share_bytes, long long plane, long long row_off, int pitch,
-                        int side, unsigned char* __restrict__ buf) {
+                        int share_bytes, const float* __restrict__ kf, long long plane,
+                        long long row_off, int pitch, int side, unsigned char* __restrict__ buf) {
   Real* out = (Real*)buf;
+  unsigned char* tail = buf + 3 * (size_t)pitch * sizeof(Real);
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < pitch; i += gridDim.x * blockDim.x) {
     for (int k = 0; k < 3; ++k) out[k * pitch + i] = f[plane_of(side, k) * plane + row_off + i];
     if (share_bytes) {
       const unsigned long long* sh = (const unsigned long long*)share;
-      ((unsigned long long*)(buf + 3 * (size_t)pitch * sizeof(Real)))[i] = sh[row_off + i];
+      ((unsigned long long*)tail)[i] = sh[row_off + i];
     }
+    if (kf) ((float*)(tail + (size_t)pitch * share_bytes))[i] = kf[row_off + i];
   }
 }
 
@@ -63,16 +66,18 @@ __global__ void k_pack0(const Real* __restrict__ f, const void* __restrict__ sha
 // neighbour across S sent its N message (planes 2, 5, 6) and vice versa.
 template <typename Real>
 __global__ void k_unpack0(Real* __restrict__ f, void* __restrict__ share, int share_bytes,
-                          long long plane, long long row_off, int pitch, int side,
-                          const unsigned char* __restrict__ buf) {
+                          float* __restrict__ kf, long long plane, long long row_off, int pitch,
+                          int side, const unsigned char* __restrict__ buf) {
   const Real* in = (const Real*)buf;
+  const unsigned char* tail = buf + 3 * (size_t)pitch * sizeof(Real);
   const int from = side == LBM_SIDE_S ? LBM_SIDE_N : LBM_SIDE_S;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < pitch; i += gridDim.x * blockDim.x) {
     for (int k = 0; k < 3; ++k) f[plane_of(from, k) * plane + row_off + i] = in[k * pitch + i];
     if (share_bytes) {
       unsigned long long* sh = (unsigned long long*)share;
-      sh[row_off + i] = ((const unsigned long long*)(buf + 3 * (size_t)pitch * sizeof(Real)))[i];
+      sh[row_off + i] = ((const unsigned long long*)tail)[i];
     }
+    if (kf) kf[row_off + i] = ((const float*)(tail + (size_t)pitch * share_bytes))[i];
   }
 }
 
@@ -139,6 +144,11 @@ long long ghost_row(const lbm_ctx* c, int side) {
   return (long long)(side == LBM_SIDE_S ? 0 : kYO + c->p.ny) * c->pitch;
 }
 
+// The rate field whose rows go with the shares, or null.
+float* shared_rates(const lbm_ctx* c) {
+  return c->p.dissolution && c->esize == 4 ? (float*)c->kf : nullptr;
+}
+
 }  // namespace
 
 extern "C" {
@@ -148,7 +158,9 @@ lbm_status lbm_halo_bytes(lbm_ctx* c, int phase, size_t* bytes) {
   if (chk != LBM_OK) return chk;
   if (!bytes || (phase != 0 && phase != 1)) return ctx_fail(LBM_ERR_ARG, "lbm_halo_bytes: bad arguments");
   const size_t P = (size_t)c->pitch;
-  *bytes = phase == 0 ? 3 * P * c->esize + (c->p.dissolution ? P * 8 : 0) : P * 4;
+  *bytes = phase == 0 ? 3 * P * c->esize + (c->p.dissolution ? P * 8 : 0) +
+                             (shared_rates(c) ? P * sizeof(float) : 0)
+                       : P * 4;
   return LBM_OK;
 }
 
@@ -162,11 +174,11 @@ lbm_status lbm_halo_pack(lbm_ctx* c, int side, int phase, void* buf) {
     const int sb = c->p.dissolution ? 8 : 0;
     if (c->esize == 8)
       k_pack0<double><<<grid, 256, 0, c->stream>>>((const double*)c->f[c->cur], c->ureact, sb,
-                                                   c->plane, row, c->pitch, side,
+                                                   nullptr, c->plane, row, c->pitch, side,
                                                    (unsigned char*)buf);
     else
       k_pack0<float><<<grid, 256, 0, c->stream>>>((const float*)c->f[c->cur], c->ureact, sb,
-                                                  c->plane, row, c->pitch, side,
+                                                  shared_rates(c), c->plane, row, c->pitch, side,
                                                   (unsigned char*)buf);
   } else {
     k_pack1<<<grid, 256, 0, c->stream>>>(c->link, row, c->pitch, (uint32_t*)buf);
@@ -184,11 +196,11 @@ lbm_status lbm_halo_unpack(lbm_ctx* c, int side, int phase, const void* buf) {
     const int sb = c->p.dissolution ? 8 : 0;
     if (c->esize == 8)
       k_unpack0<double><<<grid, 256, 0, c->stream>>>((double*)c->f[c->cur], c->ureact, sb,
-                                                     c->plane, ghost_row(c, side), c->pitch,
+                                                     nullptr, c->plane, ghost_row(c, side), c->pitch,
                                                      side, (const unsigned char*)buf);
     else
       k_unpack0<float><<<grid, 256, 0, c->stream>>>((float*)c->f[c->cur], c->ureact, sb,
-                                                    c->plane, ghost_row(c, side), c->pitch,
+                                                    shared_rates(c), c->plane, ghost_row(c, side), c->pitch,
                                                     side, (const unsigned char*)buf);
   } else {
     k_unpack1<<<1, 1024, 0, c->stream>>>(c->link, ghost_row(c, side), boundary_row(c, side),
