@@ -682,16 +682,16 @@ __device__ __forceinline__ double mineral_take(const double* __restrict__ r, lon
 // runs FP64 at 1/64 of the FP32 rate, so the terms and their sum are formed
 // in double-float arithmetic on the FP32 pipe -- T as an unevaluated float
 // pair, each product by Dekker's splitting with a fused multiply-add, the
-// sum by Knuth's two-sum -- carrying about 48 significant bits (relative
+// sum by Knuth's two-sum, each operation named so that none is merged -- carrying about 48 significant bits (relative
 // error near 1e-14), and only the final sum is converted and scaled by k in
 // FP64.  With a rate field each term is scaled in FP64.
 struct F2 {
   float hi, lo;
 };
 __device__ __forceinline__ void two_sum_add(float& s, float& e, float a) {
-  const float t = s + a;
-  const float bp = t - s;
-  e += (s - (t - bp)) + (a - bp);
+  const float t = __fadd_rn(s, a);
+  const float bp = __fsub_rn(t, s);
+  e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(a, bp)));
   s = t;
 }
 __device__ __forceinline__ double mineral_take(const ShareF32* __restrict__ sh, long long n,
@@ -720,10 +720,10 @@ __device__ __forceinline__ double mineral_take(const ShareF32* __restrict__ sh, 
                                   d.status, kSiteShare);
       const ShareF32 v = sh[s];
       const F2 t = tf[(j >= 5 ? 21 : 0) + (int)dbg_idx(v.w36, 21, d.status, kSiteShare)];
-      const float p = v.u * t.hi;
-      const float err = fmaf(v.u, t.hi, -p) + v.u * t.lo;  // u T - p, to ~2^-48 of u T
+      const float p = __fmul_rn(v.u, t.hi);
+      const float err = __fmaf_rn(v.u, t.lo, __fmaf_rn(v.u, t.hi, -p));  // u T - p, to ~2^-48 of u T
       two_sum_add(S, E, p);
-      E += err;
+      E = __fadd_rn(E, err);
     }
   return ((double)S + (double)E) * d.k_scalar;
 }

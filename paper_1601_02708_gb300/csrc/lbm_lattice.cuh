@@ -533,25 +533,28 @@ __device__ int maxent_wall_general(Real (&f)[9], unsigned solid) {
 
 // Double-float arithmetic: an unevaluated pair hi + lo carrying about 48
 // significant bits on the FP32 pipe (Dekker's products by a fused
-// multiply-add, Knuth's two-sum).
+// multiply-add, Knuth's two-sum).  The operations are named one by one: a
+// product that the compiler merged into a neighbouring sum would have its
+// rounding error, which the low part holds already, counted twice.
 struct Df {
   float hi, lo;
 };
 __device__ __forceinline__ Df df_norm(float p, float e) {  // |e| <= |p|
-  const float s = p + e;
-  return Df{s, e - (s - p)};
+  const float s = __fadd_rn(p, e);
+  return Df{s, __fsub_rn(e, __fsub_rn(s, p))};
 }
 __device__ __forceinline__ Df df_mul(Df a, Df b) {
-  const float p = a.hi * b.hi;
-  return df_norm(p, fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, fmaf(a.hi, b.hi, -p))));
+  const float p = __fmul_rn(a.hi, b.hi);
+  return df_norm(p, __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.lo, b.hi, __fmaf_rn(a.hi, b.hi, -p))));
 }
 __device__ __forceinline__ Df df_mul(Df a, float b) {
-  const float p = a.hi * b;
-  return df_norm(p, fmaf(a.lo, b, fmaf(a.hi, b, -p)));
+  const float p = __fmul_rn(a.hi, b);
+  return df_norm(p, __fmaf_rn(a.lo, b, __fmaf_rn(a.hi, b, -p)));
 }
 __device__ __forceinline__ Df df_add(Df a, Df b) {
-  const float s = a.hi + b.hi, bb = s - a.hi;
-  return df_norm(s, ((a.hi - (s - bb)) + (b.hi - bb)) + (a.lo + b.lo));
+  const float s = __fadd_rn(a.hi, b.hi), bb = __fsub_rn(s, a.hi);
+  return df_norm(s, __fadd_rn(__fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, bb)), __fsub_rn(b.hi, bb)),
+                              __fadd_rn(a.lo, b.lo)));
 }
 __host__ __device__ constexpr Df df_const(double v) { return Df{(float)v, (float)(v - (double)(float)v)}; }
 
@@ -631,17 +634,18 @@ __device__ __forceinline__ bool wall_root(const WallPoly& w, Df T, WallValues<fl
     const Df p = df_add(df_add(df_mul(pa, w.ka), df_mul(pb, w.kb)),
                         df_add(df_mul(all, w.ks), df_mul(r, w.kd)));
     const float dp = (w.ka * a * pa.hi + w.kb * b * pb.hi) + (w.ks * s * all.hi + w.kd * d * r.hi);
-    const float delta = ((C.hi - p.hi) + (C.lo - p.lo)) / dp;
+    const float delta =
+        __fadd_rn(__fsub_rn(C.hi, p.hi), __fsub_rn(C.lo, p.lo)) / dp;
     if (!(fabsf(delta) <= 4e-6f)) {
       t *= 1.f + delta;
       if (!(t > 0.f) || !isfinite(t)) return false;
       continue;
     }
     auto value = [&](Df pw, float e, Df k) {  // k pw (1 + delta)^e to second order
-      const float f = pw.hi * k.hi;
-      const float lo = fmaf(pw.hi, k.lo, fmaf(pw.lo, k.hi, fmaf(pw.hi, k.hi, -f)));
+      const float f = __fmul_rn(pw.hi, k.hi);
+      const float lo = __fmaf_rn(pw.hi, k.lo, __fmaf_rn(pw.lo, k.hi, __fmaf_rn(pw.hi, k.hi, -f)));
       const float c = e * delta;
-      return f + fmaf(f, fmaf(0.5f * (c - delta), c, c), lo);
+      return __fadd_rn(f, __fmaf_rn(f, fmaf(0.5f * (c - delta), c, c), lo));
     };
     v.a = value(pa, a, kAxis);
     v.b = value(pb, b, kAxis);
@@ -743,9 +747,9 @@ __device__ __forceinline__ int maxent_wall(Real (&f)[9], unsigned solid) {
       } else if constexpr (sizeof(Real) == 8) {
         T -= (double)d * f[i];
       } else {
-        const float p = (float)-d * f[i], e = fmaf((float)-d, f[i], -p);
-        const float s = Th + p, bb = s - Th;
-        Tl += ((Th - (s - bb)) + (p - bb)) + e;
+        const float p = __fmul_rn((float)-d, f[i]), e = __fmaf_rn((float)-d, f[i], -p);
+        const float s = __fadd_rn(Th, p), bb = __fsub_rn(s, Th);
+        Tl = __fadd_rn(Tl, __fadd_rn(__fadd_rn(__fsub_rn(Th, __fsub_rn(s, bb)), __fsub_rn(p, bb)), e));
         Th = s;
       }
     }
