@@ -715,6 +715,18 @@ __device__ __noinline__ int maxent_wall_rare(Real* f, unsigned solid) {
   return r;
 }
 
+// sum_{others} (e_j.m) f_j in FP64 (out of line: a wall whose flux cancels is rare)
+static __device__ __noinline__ double wall_flux(float f1, float f2, float f3, float f4, float f5,
+                                                float f6, float f7, float f8, unsigned neg, int mx,
+                                                int my) {
+  const float f[9] = {0.f, f1, f2, f3, f4, f5, f6, f7, f8};
+  double T = 0.0;
+#pragma unroll
+  for (int i = 1; i < 9; ++i)
+    if (!(neg & (1u << i))) T += (double)(cx_of(i) * mx + cy_of(i) * my) * (double)f[i];
+  return T;
+}
+
 template <typename S, typename Real>
 __device__ __forceinline__ int maxent_wall(Real (&f)[9], unsigned solid) {
   if constexpr (sizeof(S) == 4) {
@@ -734,7 +746,7 @@ __device__ __forceinline__ int maxent_wall(Real (&f)[9], unsigned solid) {
     // T = sum_{others} (e_j.m) f_j: integer multiples of the populations,
     // summed in FP64, or in double-float for FP32 populations
     double T = 0.0;
-    float Th = 0.f, Tl = 0.f;
+    float Th = 0.f, Tl = 0.f, most = 0.f;
 #pragma unroll
     for (int i = 1; i < 9; ++i) {
       const int d = -(cx_of(i) * mx + cy_of(i) * my);
@@ -751,10 +763,20 @@ __device__ __forceinline__ int maxent_wall(Real (&f)[9], unsigned solid) {
         const float s = __fadd_rn(Th, p), bb = __fsub_rn(s, Th);
         Tl = __fadd_rn(Tl, __fadd_rn(__fadd_rn(__fsub_rn(Th, __fsub_rn(s, bb)), __fsub_rn(p, bb)), e));
         Th = s;
+        most = fmaxf(most, fabsf(p));
       }
     }
     if (!neg) return kWallSet;
-    const Df Td = df_norm(Th, Tl);
+    Df Td = df_norm(Th, Tl);
+    if constexpr (sizeof(Real) == 4) {
+      // the pair holds the sum to 2^-48 of its largest term: where less than a
+      // thousandth of that is left (or a product overflows) it is summed in FP64
+      if (most > 0.f && !(fabsf(Td.hi) > kEdgeCancel * most && most < kEdgeHigh)) {
+        T = wall_flux(f[1], f[2], f[3], f[4], f[5], f[6], f[7], f[8], neg, mx, my);
+        Td.hi = (float)T;
+        Td.lo = (float)(T - (double)Td.hi);
+      }
+    }
     const Real size = sizeof(Real) == 8 ? (Real)T : (Real)Td.hi;
     if (!(size > (Real)0)) {
 #pragma unroll

@@ -123,3 +123,49 @@ def test_side_solves(gb, kernel):
                 assert abs(got[i, y, x] - want) <= ULP * want
             for i in known[1:]:
                 assert got[i, y, x] == g[i, y, x]
+
+
+# One solid node beside a fluid one: the side it lies on, and the populations of
+# the flux sum in the order of their directions.  Terms near one and near 2^-25
+# cancel, and what is left is below 2^-48 of the largest.
+CANCEL = [
+    ("E", ["0x1.00001p-24", "0x1p+0", "0x1p+0", "0x1.00001p-24", "0x1p-49"]),
+    ("W", ["0x1p+0", "0x1p-50", "0x1.7ffff6p-4", "0x1.4p-25", "0x1.18p+0"]),
+    ("N", ["0x1.4p-49", "0x1.0008p+0", "0x1.fff00cp-1", "0x1.000004p+0", "0x1.000002p+0"]),
+    ("S", ["0x1p-51", "0x1p-26", "0x1.00004p+0", "0x1p+0", "0x1.01p-18"]),
+]
+
+
+@pytest.mark.parametrize("kernel", ["tma", "generic"])
+def test_wall_flux_that_cancels(gb, kernel):
+    """The root, and whether there is one, where the flux sum cancels."""
+    nx, ny = 64, 40
+    to = {"E": (1, 0), "W": (-1, 0), "N": (0, 1), "S": (0, -1)}
+    solid = np.zeros((ny, nx), bool)
+    f = np.full((9, ny, nx), 0.5, np.float32)
+    nodes = []
+    for k, (side, values) in enumerate(CANCEL):
+        x, y, (sx, sy) = 8 + 12 * k, 20, to[side]
+        solid[y + sy, x + sx] = True
+        nodes.append((x, y))
+        terms = [i for i in range(1, 9) if C[i][0] * sx + C[i][1] * sy and C[i] != (-sx, -sy)]
+        for i, v in zip(terms, values):
+            f[i, y - C[i][1], x - C[i][0]] = float.fromhex(v)
+    f *= ~solid
+    lat = gb.LBM(nx, ny, 1e30, solid=solid, vel=np.zeros((2, ny, nx)), u0=np.zeros((ny, nx)), walls="maxent")
+    lat.set_kernel(kernel)
+    with_populations(lat, f).substeps(1, 1)
+    got, (g, up) = lat.populations(), streamed(f, solid)
+    noroot = 0
+    for y, x in zip(*np.nonzero(~solid)):
+        link = [i for i in range(1, 9) if up[i, y, x]]
+        want, T = wall_solve(g[:, y, x], link) if link else ({}, 0)
+        noroot += T < 0
+        if (x, y) in nodes:
+            assert 0 < abs(T) < 1e-14
+        for i, v in want.items():
+            if T > 0:
+                assert abs(got[i, y, x] - v) <= ULP * v
+            else:  # zero, and what the collision adds: w u / tau
+                assert 0 <= got[i, y, x] <= 1e-30
+    assert lat.diagnostics()["bc_infeasible"] == noroot == 1
