@@ -104,3 +104,12 @@ bool ctx_on_this_device(const void* p, int device) {
   }
   return at.type == cudaMemoryTypeDevice && at.device == device;
 }
+
+bool ctx_in_reach(const void* p, int device) {
+  cudaPointerAttributes at;
+  if (!p || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeManaged || (at.type == cudaMemoryTypeDevice && at.device == device);
+}

@@ -139,6 +139,9 @@ lbm_status ctx_status(lbm_ctx* c);   // waits for the stream, reads the device e
 bool ctx_on_device(const void* p);
 // Memory of this kind and device: what ctx_copy_list may read and write.
 bool ctx_on_this_device(const void* p, int device);
+// Memory that a kernel on the device may read and write in place: the device's
+// own or managed, not another device's (ctx_on_device holds for that too).
+bool ctx_in_reach(const void* p, int device);
 // Copies within the device, one launch for up to kCopyMax of them (lbm_copy.cu);
 // a null source is zeros.  The regions do not overlap.  `head`, at most
 // kCopyHead bytes of host memory, is written to head_dst with the first launch

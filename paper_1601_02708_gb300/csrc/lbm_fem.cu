@@ -831,6 +831,7 @@ struct lbm_fem {
   long long n = 0;
   int n_dir = 0;
   cudaStream_t stream = nullptr;
+  int device = 0;
   double* A = nullptr;  // [9][n]
   double* B = nullptr;  // [9][n]
   double* d = nullptr;  // state
@@ -1046,6 +1047,7 @@ lbm_status lbm_fem_init(lbm_fem** out, const lbm_fem_params* p, const uint8_t* e
   {
     int dev = 0, sms = 0, coop = 0, per_sm = 0;
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    f->device = dev;
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
     if (e == cudaSuccess)
@@ -1097,9 +1099,9 @@ lbm_status lbm_fem_step(lbm_fem* f, const double* dir_values) {
   cudaStream_t s = f->stream;
   const double* fixed = f->fixed_val;
   if (f->n_dir > 0) {
-    if (ctx_on_device(dir_values)) fixed = dir_values;  // read in place: this call waits
+    if (ctx_in_reach(dir_values, f->device)) fixed = dir_values;  // read in place: this call waits
     else FCK(cudaMemcpyAsync(f->fixed_val, dir_values, f->n_dir * sizeof(double),
-                             cudaMemcpyHostToDevice, s));
+                             cudaMemcpyDefault, s));
   }
   Outcome& h = *f->pinned;
   h = Outcome{};

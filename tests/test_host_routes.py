@@ -1,0 +1,31 @@
+"""Which memory the library's host code hands to kernels and which it copies:
+memory of another device is copied, not dereferenced.  On a recording stand-in
+for the CUDA runtime (no GPU, kernels not run)."""
+import ctypes
+
+import pytest
+
+import fake_cuda
+from fake_cuda import DEVICE, HOST, MANAGED
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    return fake_cuda.load(str(tmp_path_factory.mktemp("fake")))
+
+
+@pytest.mark.parametrize("kind,device,copied", [(DEVICE, 0, False), (MANAGED, 0, False),
+                                                (DEVICE, 1, True), (HOST, 0, True)])
+@pytest.mark.parametrize("nex,ney", [(20, 10), (700, 330)])  # by tiles, over all nodes
+def test_dirichlet_values_of_a_continuum_step(fake, nex, ney, kind, device, copied):
+    from paper_1601_02708_gb300._lib import FemParams
+    p = FemParams(nex=nex, ney=ney, hx=0.1, hy=0.1, D=1.0, theta=0.5, dt=0.1)
+    nodes = (ctypes.c_int * 5)(*range(5))
+    h = ctypes.c_void_p()
+    assert fake.lib.lbm_fem_init(ctypes.byref(h), ctypes.byref(p), None, 5, nodes, None, None) == 0
+    vals = fake.buffer(5 * 8, kind, device)
+    fake.clear()
+    fake.lib.lbm_fem_step(h, vals)  # (no kernel runs: it reports no convergence)
+    assert fake.launched("k_bicgstab_tile" if nex < 100 else "k_bicgstab")
+    assert any(s == ctypes.addressof(vals) and n == 40 for _, s, n in fake.copies()) == copied
+    fake.lib.lbm_fem_destroy(h)
