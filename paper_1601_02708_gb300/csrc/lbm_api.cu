@@ -802,18 +802,18 @@ static_assert(sizeof(BlobHeader) <= 64 && sizeof(BlobHeader) <= kCopyHead, "the 
 template <typename T, typename O>
 lbm_status field_out(lbm_ctx* c, const T* src, O* dst, int planes) {
   const size_t bytes = (size_t)planes * c->p.nx * c->p.ny * sizeof(O);
-  const bool dev = on_device(dst);
+  const bool direct = ctx_in_reach(dst, c->device);  // (memory of another device is copied to)
   O* d = dst;
-  if (!dev) {
+  if (!direct) {
     TRY(ensure_scratch(c, bytes));
     d = (O*)c->scratch;
   }
   k_pitch_out<T, O><<<grid1d((long long)planes * c->p.nx * c->p.ny), 256, 0, c->stream>>>(
       src, d, c->p.nx, c->p.ny, c->pitch, planes);
   CK(cudaGetLastError());
-  if (!dev) {
-    CK(cudaMemcpyAsync(dst, d, bytes, cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
+  if (!direct) {
+    CK(cudaMemcpyAsync(dst, d, bytes, cudaMemcpyDefault, c->stream));
+    if (!on_device(dst)) CK(cudaStreamSynchronize(c->stream));
   }
   return LBM_OK;
 }

@@ -29,3 +29,22 @@ def test_dirichlet_values_of_a_continuum_step(fake, nex, ney, kind, device, copi
     assert fake.launched("k_bicgstab_tile" if nex < 100 else "k_bicgstab")
     assert any(s == ctypes.addressof(vals) and n == 40 for _, s, n in fake.copies()) == copied
     fake.lib.lbm_fem_destroy(h)
+
+
+@pytest.mark.parametrize("kind,device,copied", [(DEVICE, 0, False), (MANAGED, 0, False),
+                                                (DEVICE, 1, True), (HOST, 0, True)])
+@pytest.mark.parametrize("what", ["lbm_get_populations", "lbm_adjoint"])
+def test_fields_read_out(fake, what, kind, device, copied):
+    """(outlet_breakthrough reads dJ/dk into memory where its rate field is)"""
+    h = fake.lattice(40, 30)
+    out = fake.buffer(9 * 40 * 30 * 8, kind, device)
+    fake.clear()
+    if what == "lbm_adjoint":
+        bytes_ = 40 * 30 * 8
+        st = fake.lib.lbm_adjoint(h, 2, 1, 0, None, None, None, None, out, None, None, None, None)
+    else:
+        bytes_ = 9 * 40 * 30 * 8
+        st = fake.lib.lbm_get_populations(h, out)
+    assert st == 0
+    assert any(d == ctypes.addressof(out) and n == bytes_ for d, _, n in fake.copies()) == copied
+    fake.lib.lbm_destroy(h)
