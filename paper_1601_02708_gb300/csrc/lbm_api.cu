@@ -1275,15 +1275,18 @@ lbm_status lbm_save(lbm_ctx* c, void* buf, size_t bytes) {
     CK(ctx_copy_list(items, n, c->stream, &h, buf, (int)sizeof(h)));
     return LBM_OK;
   }
-  // host memory, or memory that this device does not hold
+  // host memory, managed memory, or another device's, where a kernel cannot
+  // put the header
   const cudaMemcpyKind k = dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-  if (dev) CK(cudaMemcpyAsync(buf, &h, sizeof(h), cudaMemcpyDefault, c->stream));
+  const bool reach = ctx_in_reach(buf, c->device);
+  if (reach) CK(ctx_copy_list(nullptr, 0, c->stream, &h, buf, (int)sizeof(h)));
+  else if (dev) CK(cudaMemcpyAsync(buf, &h, sizeof(h), cudaMemcpyDefault, c->stream));
   else memcpy(buf, &h, sizeof(h));
   for (int i = 0; i < n; ++i) {
     CK(cudaMemcpyAsync((char*)buf + off, s[i].ptr, s[i].bytes, k, c->stream));
     off += align256(s[i].bytes);
   }
-  if (dev) CK(cudaStreamSynchronize(c->stream));
+  if (dev && !reach) CK(cudaStreamSynchronize(c->stream));
   if (dev) return LBM_OK;
   return check_status(c);  // waits: the host blob is complete on return
 }

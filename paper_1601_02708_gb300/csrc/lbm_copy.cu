@@ -44,6 +44,7 @@ __device__ __forceinline__ void move_as(char* dst, const char* src, size_t len) 
 // together, with 72 pieces of edge data, from 2.58 to 2.21 ms.
 __global__ void __launch_bounds__(kCopyThreads) k_copy_list(const __grid_constant__ CopyArgs a) {
   if (blockIdx.x == 0 && (int)threadIdx.x < a.head_bytes) a.head_dst[threadIdx.x] = a.head[threadIdx.x];
+  if (a.n == 0) return;  // the head alone
   int i = 0;
   while (i + 1 < a.n && (int)blockIdx.x >= a.first[i + 1]) ++i;
   const CopyItem it = a.item[i];
@@ -69,10 +70,11 @@ __global__ void __launch_bounds__(kCopyThreads) k_copy_list(const __grid_constan
 cudaError_t ctx_copy_list(const CopyItem* items, int n, cudaStream_t stream, const void* head,
                           void* head_dst, int head_bytes) {
   int k = 0;
-  while (k < n) {
+  bool headed = head_bytes == 0;
+  while (k < n || !headed) {
     CopyArgs a;
     a.n = 0;
-    a.head_bytes = k == 0 ? head_bytes : 0;
+    a.head_bytes = headed ? 0 : head_bytes;
     a.head_dst = (unsigned char*)head_dst;
     if (a.head_bytes) memcpy(a.head, head, (size_t)head_bytes);
     long long blocks = 0;
@@ -84,12 +86,11 @@ cudaError_t ctx_copy_list(const CopyItem* items, int n, cudaStream_t stream, con
       a.first[a.n++] = (int)blocks;
       blocks += need;
     }
-    if (a.n == 0) {
-      if (k < n) return cudaErrorInvalidValue;
-      break;
-    }
+    if (a.n == 0 && k < n) return cudaErrorInvalidValue;
+    if (a.n == 0 && headed) break;
+    headed = true;
     a.first[a.n] = (int)blocks;
-    k_copy_list<<<(unsigned)blocks, kCopyThreads, 0, stream>>>(a);
+    k_copy_list<<<(unsigned)(blocks > 0 ? blocks : 1), kCopyThreads, 0, stream>>>(a);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }

@@ -48,3 +48,19 @@ def test_fields_read_out(fake, what, kind, device, copied):
     assert st == 0
     assert any(d == ctypes.addressof(out) and n == bytes_ for d, _, n in fake.copies()) == copied
     fake.lib.lbm_destroy(h)
+
+
+@pytest.mark.parametrize("kind,device,waits", [(DEVICE, 0, 0), (MANAGED, 0, 0), (DEVICE, 1, 1)])
+def test_save_into_device_memory(fake, kind, device, waits):
+    """It queues copies and returns, so that it can be captured; the header does
+    not travel from the call's stack unless the call waits (another device)."""
+    h = fake.lattice(40, 30)
+    n = fake.state_bytes(h)
+    blob = fake.buffer(n, kind, device)
+    fake.clear()
+    fake.lib.lbm_save.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_size_t]
+    assert fake.lib.lbm_save(h, blob, n) == 0
+    assert fake.waits() == waits
+    header = any(d == ctypes.addressof(blob) for d, _, _ in fake.copies())
+    assert header == (waits > 0) and fake.launched("k_copy_list") == (waits == 0)
+    fake.lib.lbm_destroy(h)
