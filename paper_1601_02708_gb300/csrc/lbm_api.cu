@@ -556,6 +556,21 @@ lbm_status setup_tma(lbm_ctx* c) {
   return LBM_OK;
 }
 
+// Partials of a lattice: one per block of the generic kernel (of this many rows),
+// and enough for a batch's pipelined tiles plus its boundary-warp chunks of 32
+// nodes.  A lattice holds those of the smallest blocks whichever it runs: which
+// ones an FP64 lattice runs depends on the device's SMs, and saved states hold the
+// partials, whose number must not.
+int partials_of(const lbm_ctx* c, int rows) {
+  const lbm_params& p = c->p;
+  const long long generic =
+      (long long)((p.nx + lbm::kBX - 1) / lbm::kBX) * ((p.ny + rows - 1) / rows);
+  const long long tiles = (long long)((p.nx + lbm::kTW - 1) / lbm::kTW) *
+                          ((p.ny + lbm::kTH - 1) / lbm::kTH) + (c->n_open + 31) / 32;
+  return (int)((generic > tiles ? generic : tiles) + 1);
+}
+static_assert(lbm::step_rows<float>() == lbm::kSmallRows, "FP32 lattices hold as many in every state");
+
 lbm_status init_impl(lbm_ctx* c, const uint8_t* solid, const double* vel,
                      const double* k_field, const double* mineral, const double* u0) {
   const lbm_params& p = c->p;
@@ -650,14 +665,7 @@ lbm_status init_impl(lbm_ctx* c, const uint8_t* solid, const double* vel,
   CK(cudaMemsetAsync(c->jnode, 0, (size_t)p.ny * sizeof(double), c->stream));
   CK(cudaMalloc((void**)&c->jflux, (size_t)p.ny * sizeof(double)));
   CK(cudaMemsetAsync(c->jflux, 0, (size_t)p.ny * sizeof(double), c->stream));
-  {
-    // one partial per block of the generic kernel, and enough for a batch's
-    // pipelined tiles plus its boundary-warp chunks of 32 nodes
-    const long long generic = (long long)c->sgrid.x * c->sgrid.y;
-    const long long tiles = (long long)((p.nx + lbm::kTW - 1) / lbm::kTW) *
-                            ((p.ny + lbm::kTH - 1) / lbm::kTH) + (c->n_open + 31) / 32;
-    c->partial_cap = (int)((generic > tiles ? generic : tiles) + 1);
-  }
+  c->partial_cap = partials_of(c, lbm::kSmallRows);
   CK(cudaMalloc((void**)&c->partial, (size_t)c->partial_cap * sizeof(double)));
   CK(cudaMemsetAsync(c->partial, 0, (size_t)c->partial_cap * sizeof(double), c->stream));
   CK(cudaMalloc((void**)&c->diag, sizeof(DiagDev)));
@@ -767,7 +775,8 @@ struct Section {
   void* ptr;
   size_t bytes;
 };
-int state_sections(lbm_ctx* c, Section* s) {
+// (partials: those the state holds, see state_partials)
+int state_sections(lbm_ctx* c, Section* s, int partials) {
   int k = 0;
   const size_t plane_b = (size_t)c->plane * c->esize;
   s[k++] = {c->f[c->cur], 9 * plane_b};
@@ -775,7 +784,7 @@ int state_sections(lbm_ctx* c, Section* s) {
   s[k++] = {c->u, plane_b};
   s[k++] = {c->infeasible, (size_t)c->nedge * sizeof(long long)};
   s[k++] = {c->jnode, (size_t)c->p.ny * sizeof(double)};
-  s[k++] = {c->partial, (size_t)c->partial_cap * sizeof(double)};
+  s[k++] = {c->partial, (size_t)partials * sizeof(double)};
   s[k++] = {c->jflux, (size_t)c->p.ny * sizeof(double)};
   s[k++] = {c->counters, 4 * sizeof(long long)};
   if (c->p.dissolution) {
@@ -794,7 +803,28 @@ struct BlobHeader {
   long long steps;
   int nx, ny, precision, dissolution, nparts, pad;
 };
-const unsigned long long kMagic = 0x4C424D4144453035ull;  // "LBMADE05"
+const unsigned long long kMagic = 0x4C424D4144453036ull;     // "LBMADE06"
+const unsigned long long kMagicOld = 0x4C424D4144453035ull;  // "LBMADE05": see state_partials
+size_t state_size(lbm_ctx* c, int partials) {
+  Section s[16];
+  const int k = state_sections(c, s, partials);
+  size_t total = align256(sizeof(BlobHeader));
+  for (int i = 0; i < k; ++i) total += align256(s[i].bytes);
+  return total;
+}
+
+// Partials that a state of this header holds, in a buffer of this many bytes.
+// States of the earlier form hold those of the blocks the lattice ran: on the
+// FP32 lattice as many as now, on the FP64 lattice those of 32 x 8 blocks, or of
+// 32 x 2 blocks where the lattice was small for its device, which shows in the
+// number it left or, before the first step, in the size of the buffer.
+int state_partials(lbm_ctx* c, const BlobHeader& h, size_t bytes) {
+  if (h.magic == kMagic || c->esize == 4) return c->partial_cap;
+  const int few = partials_of(c, lbm::step_rows<double>());
+  if (h.nparts > few) return c->partial_cap;
+  const bool small = (int)c->sblock.y == lbm::kSmallRows;
+  return small && bytes >= state_size(c, c->partial_cap) ? c->partial_cap : few;
+}
 static_assert(sizeof(BlobHeader) <= 64 && sizeof(BlobHeader) <= kCopyHead, "the header fits its pinned read-back slot");
 
 // Copy a padded device field out to a caller array (host or device) of
@@ -1246,11 +1276,7 @@ lbm_status lbm_get_flip_steps(lbm_ctx* c, int32_t* out) {
 lbm_status lbm_state_bytes(lbm_ctx* c, size_t* bytes) {
   TRY(check_ctx(c));
   if (!bytes) return fail(LBM_ERR_ARG, "lbm_state_bytes: null out");
-  Section s[16];
-  const int k = state_sections(c, s);
-  size_t total = align256(sizeof(BlobHeader));
-  for (int i = 0; i < k; ++i) total += align256(s[i].bytes);
-  *bytes = total;
+  *bytes = state_size(c, c->partial_cap);
   return LBM_OK;
 }
 
@@ -1262,7 +1288,7 @@ lbm_status lbm_save(lbm_ctx* c, void* buf, size_t bytes) {
   TRY(sync_mineral(c));
   BlobHeader h{kMagic, c->steps, c->p.nx, c->p.ny, c->p.precision, c->p.dissolution, c->nparts, 0};
   Section s[16];
-  const int n = state_sections(c, s);
+  const int n = state_sections(c, s, c->partial_cap);
   size_t off = align256(sizeof(BlobHeader));
   if (ctx_on_this_device(buf, c->device)) {
     // one launch; the header travels as a kernel argument: nothing on this
@@ -1292,9 +1318,9 @@ lbm_status lbm_save(lbm_ctx* c, void* buf, size_t bytes) {
 }
 
 lbm_status lbm_restore(lbm_ctx* c, const void* buf, size_t bytes) {
-  size_t need = 0;
-  TRY(lbm_state_bytes(c, &need));
-  if (!buf || bytes < need) return fail(LBM_ERR_ARG, "lbm_restore: buffer smaller than lbm_state_bytes");
+  TRY(check_ctx(c));
+  const int fewest = c->esize == 8 ? partials_of(c, lbm::step_rows<double>()) : c->partial_cap;
+  if (!buf || bytes < state_size(c, fewest)) return fail(LBM_ERR_ARG, "lbm_restore: buffer smaller than lbm_state_bytes");
   const bool dev = on_device(buf);
   BlobHeader h;
   if (dev) {
@@ -1306,11 +1332,16 @@ lbm_status lbm_restore(lbm_ctx* c, const void* buf, size_t bytes) {
     CK(cudaStreamSynchronize(c->stream));  // the sections below overwrite the state
     memcpy(&h, buf, sizeof(h));
   }
-  if (h.magic != kMagic || h.nx != c->p.nx || h.ny != c->p.ny ||
+  if ((h.magic != kMagic && h.magic != kMagicOld) || h.nx != c->p.nx || h.ny != c->p.ny ||
       h.precision != c->p.precision || h.dissolution != c->p.dissolution)
     return fail(LBM_ERR_STATE, "lbm_restore: blob does not belong to this lattice");
+  const int partials = state_partials(c, h, bytes);
+  if (bytes < state_size(c, partials))
+    return fail(LBM_ERR_ARG, "lbm_restore: buffer smaller than lbm_state_bytes");
+  if (h.nparts < 0 || h.nparts > partials)
+    return fail(LBM_ERR_STATE, "lbm_restore: blob does not belong to this lattice");
   Section s[16];
-  const int n = state_sections(c, s);
+  const int n = state_sections(c, s, partials);
   size_t off = align256(sizeof(BlobHeader));
   if (ctx_on_this_device(buf, c->device)) {
     CopyItem items[16];
