@@ -1087,6 +1087,7 @@ lbm_status lbm_step_stream(lbm_ctx* c, int j, int eta, int final_step) {
   if (c->esize == 8) TRY(launch_step_impl<double>(c, step_args<double>(c, frac), final_step != 0));
   else TRY(launch_step_impl<float>(c, step_args<float>(c, frac), final_step != 0));
   TRY(time_end(c, 0));
+  c->first_pass_over = false;
   c->cur ^= 1;
   c->steps += 1;
   return LBM_OK;
@@ -1095,7 +1096,13 @@ lbm_status lbm_step_stream(lbm_ctx* c, int j, int eta, int final_step) {
 lbm_status lbm_step_dissolve(lbm_ctx* c) {
   TRY(check_ctx(c));
   if (!c->p.dissolution) return LBM_OK;
+  if (c->first_pass_over) {  // the pass that was due lies behind the restored state
+    c->first_pass_over = false;
+    return LBM_OK;
+  }
   if (c->first_pass_due) {
+    // (a restored state's word [1] is the list's length: open_pass)
+    CK(cudaMemsetAsync(c->flip_count + 1, 0, sizeof(int), c->stream));
     TRY(c->esize == 8 ? first_dissolve<double>(c) : first_dissolve<float>(c));
     c->first_pass_due = false;
     return LBM_OK;
@@ -1343,6 +1350,16 @@ lbm_status lbm_restore(lbm_ctx* c, const void* buf, size_t bytes) {
   Section s[16];
   const int n = state_sections(c, s, partials);
   size_t off = align256(sizeof(BlobHeader));
+  const bool fresh = c->first_pass_due || c->first_pass_over;
+  int passes = 0;  // dissolution passes the state has behind it
+  if (fresh) {
+    size_t at = off;
+    for (int i = 0; i < n && s[i].ptr != c->flip_count; ++i) at += align256(s[i].bytes);
+    int* words = (int*)((char*)c->pinned + 128);
+    CK(cudaMemcpyAsync(words, (const char*)buf + at, 4 * sizeof(int), cudaMemcpyDefault, c->stream));
+    CK(cudaStreamSynchronize(c->stream));
+    passes = words[3];
+  }
   if (ctx_on_this_device(buf, c->device)) {
     CopyItem items[16];
     for (int i = 0; i < n; ++i) {
@@ -1367,6 +1384,10 @@ lbm_status lbm_restore(lbm_ctx* c, const void* buf, size_t bytes) {
         c->link, (unsigned long long*)c->ureact, c->p.nx, c->p.ny, c->pitch,
         c->p.edge[0] == LBM_EDGE_PERIODIC, c->p.edge[2] == LBM_EDGE_PERIODIC, c->plane, c->status);
     CK(cudaGetLastError());
+  }
+  if (fresh) {  // a slab that has not stepped: is its first pass due in this state?
+    c->first_pass_due = passes == 0;
+    c->first_pass_over = passes > 0;
   }
   c->steps = h.steps;
   c->nparts = h.nparts;

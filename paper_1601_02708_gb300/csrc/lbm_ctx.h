@@ -41,6 +41,7 @@ struct lbm_ctx {
   // unsplit lattice has y0 = 0, ny_global = p.ny.
   int y0 = 0, ny_global = 0, per_y_global = 0;
   bool first_pass_due = false;  // the first dissolution pass waits for the halo
+  bool first_pass_over = false;  // it was due when a state past it was restored
   int pitch = 0;
   long long plane = 0;  // pitch * rows
   size_t esize = 4;

@@ -71,3 +71,19 @@ def test_between_the_halves_of_a_step(gb, edges, precision, where):
         lat.close()
     assert all(np.array_equal(a, b) for a, b in zip(*runs))
     assert (runs[0][-1] >= 0).any()
+
+
+@pytest.mark.parametrize("precision", [32, 64])
+def test_run_resumed_in_fresh_slabs(gb, precision):
+    """A run's states restored into slabs that have not stepped: they go on as it does."""
+    from paper_1601_02708_gb300.partition import SlabLattice
+    ud = np.ones(2 * (NX + NY))
+    kw = _case((1, 2, 0, 0))
+    run, fresh = (SlabLattice(NX, NY, 0.8, parts=3, precision=precision, **kw) for _ in range(2))
+    run.substeps(12, 1, ud, ud)
+    for a, b in zip(run.slabs, fresh.slabs):
+        b.restore(a.save())
+    for lat in (run, fresh):
+        lat.substeps(9, 1, ud, ud)
+    assert all(np.array_equal(a, b) for a, b in zip(_state(run), _state(fresh)))
+    assert run.diagnostics()["flips"] == fresh.diagnostics()["flips"] > 0

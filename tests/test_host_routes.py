@@ -64,3 +64,35 @@ def test_save_into_device_memory(fake, kind, device, waits):
     header = any(d == ctypes.addressof(blob) for d, _, _ in fake.copies())
     assert header == (waits > 0) and fake.launched("k_copy_list") == (waits == 0)
     fake.lib.lbm_destroy(h)
+
+
+@pytest.mark.parametrize("passes", [0, 5])
+def test_state_restored_into_a_fresh_slab(fake, passes):
+    """The first pass over every node starts with its block counter at zero, and
+    is not run on a state that has passes behind it."""
+    import numpy as np
+    from paper_1601_02708_gb300._lib import Params
+    p = Params(nx=40, ny=30, precision=64, tau=0.8, react_mode=1, k_scalar=0.1, dissolution=1)
+    h = ctypes.c_void_p()
+    assert fake.lib.lbm_init_slab(ctypes.byref(h), ctypes.byref(p), 0, 12, None, None, None, None, None, None) == 0
+    n = fake.state_bytes(h)
+    fake.lib.lbm_save.argtypes = fake.lib.lbm_restore.argtypes = [ctypes.c_void_p, ctypes.c_void_p,
+                                                                  ctypes.c_size_t]
+    blob = np.zeros(n, np.uint8)
+    assert fake.lib.lbm_save(h, blob.ctypes.data, n) == 0
+    up = lambda b: -(-b // 256) * 256
+    plane = 160 * 14
+    # from the end: flip steps, minerals and nodes of the surface list, the words
+    at = n - up(4 * plane) - up(8 * 480) - up(4 * 480) - 256
+    blob[at:at + 16].view(np.int32)[:] = (0, 7, 7, passes)
+    assert fake.lib.lbm_restore(h, blob.ctypes.data, n) == 0
+    fake.clear()
+    assert fake.lib.lbm_step_dissolve(h) == 0
+    assert fake.launched("lbm_dissolve_dense") == (passes == 0) and not fake.launched("lbm_dissolve_list")
+    back = np.zeros(n, np.uint8)
+    assert fake.lib.lbm_save(h, back.ctypes.data, n) == 0
+    assert list(back[at:at + 16].view(np.int32)) == [0, 0 if passes == 0 else 7, 7, passes]
+    fake.clear()
+    assert fake.lib.lbm_step_stream(h, 1, 1, 1) == 0 and fake.lib.lbm_step_dissolve(h) == 0
+    assert fake.launched("lbm_dissolve_list")
+    fake.lib.lbm_destroy(h)
