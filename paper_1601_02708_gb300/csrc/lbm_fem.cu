@@ -442,6 +442,10 @@ __host__ __device__ constexpr size_t tile_doubles(int tw, int th) {
   return 7 * ring + 11 * own + kTileVals * kTileThreads + ring + own;
 }
 
+// Exponent field of a double: 0 for zeros and numbers below the normal range,
+// 0x7ff for infinities and NaN.
+__device__ __forceinline__ int exponent(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
+
 __device__ __forceinline__ unsigned long long tile_ns() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -504,18 +508,18 @@ __device__ __forceinline__ double warp_sum(const double (&a)[N], int n) {
   unsigned top = 0;
 #pragma unroll
   for (int i = 0; i < N; ++i)
-    if (i < n) top = max(top, ((unsigned)__double2hiint(a[i]) >> 20) & 0x7ffu);
+    if (i < n) top = max(top, (unsigned)exponent(a[i]));
   top = __reduce_max_sync(kFull, top);
-  if (top == 0u) return 0.0;  // zeros (or below the normal range)
+  if (top == 0u) top = 1u;  // zeros and numbers below the normal range, in units of 2^-1074
   if (top == 0x7ffu) return __longlong_as_double(0x7ff8000000000000ll);
   long long s = 0;
 #pragma unroll
   for (int i = 0; i < N; ++i)
     if (i < n) {
       const long long b = __double_as_longlong(a[i]);
-      const int e = (int)((b >> 52) & 0x7ff), sh = (int)top - e;
-      long long m = ((b & 0xFFFFFFFFFFFFFll) | 0x10000000000000ll) << 1;
-      m = (e == 0 || sh > 54) ? 0 : (m + ((1ll << sh) >> 1)) >> sh;
+      const int e = (int)((b >> 52) & 0x7ff), sh = (int)top - (e > 0 ? e : 1);
+      long long m = ((b & 0xFFFFFFFFFFFFFll) | (e > 0 ? 0x10000000000000ll : 0ll)) << 1;
+      m = sh > 54 ? 0 : (m + ((1ll << sh) >> 1)) >> sh;
       s += b < 0 ? -m : m;
     }
   const unsigned lo = __reduce_add_sync(kFull, (unsigned)s & 0x3FFFFFFu);
@@ -739,6 +743,7 @@ __global__ void __launch_bounds__(kTileThreads) k_bicgstab_tile(const TileSolve 
     // alpha / rho = 1 / (rhat.v): the two divisions run side by side, in lanes
     // 0 and 1 of the first warp
     double rho_new = 0.0, omega_l = 0.0, per_rho = 0.0;
+    bool far = false;
     auto verdict = [&]() {  // thread 0, after rho_new and rnorm2
       ++it;
       if (dead) stop = 5;
@@ -748,12 +753,16 @@ __global__ void __launch_bounds__(kTileThreads) k_bicgstab_tile(const TileSolve 
       else {
         stop = 0;
         bc[2] = rho_new * per_rho;
+        if (far) bc[2] = rho_new / rv * per_rho;
       }
       rho = rho_new;
     };
     if (tid < 32) {
       const double rv0 = __shfl_sync(0xffffffffu, rv, 0);
-      const double q = tid == 1 ? sums[1] / (sums[0] * rv0) : sums[0] / sums[1];
+      // the product t.s rhat.v is of the data's fourth power, and out of range
+      // before their squares are: then beta = (rho_new / rhat.v) (t.t / t.s)
+      far = (unsigned)(exponent(sums[0]) + exponent(rv0) - 1023 - 64) > 1900u;
+      const double q = tid == 1 ? sums[1] / (far ? sums[0] : sums[0] * rv0) : sums[0] / sums[1];
       per_rho = __shfl_sync(0xffffffffu, q, 1);
       omega_l = sums[1] > 0.0 ? q : 0.0;
       if (lead) {
