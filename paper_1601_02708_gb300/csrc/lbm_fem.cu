@@ -769,7 +769,9 @@ __global__ void __launch_bounds__(kTileThreads) k_bicgstab_tile(const TileSolve 
         bc[1] = omega_l;
         rho_new = sums[2] - omega_l * sums[3];
         rnorm2 = sums[4] - omega_l * (2.0 * sums[0] - omega_l * sums[1]);
-        if (!(rnorm2 > 1e-10 * sums[4]) && sums[4] > 0.0) stop = 4;
+        if ((!(rnorm2 > 1e-10 * sums[4]) && sums[4] > 0.0) ||
+            exponent(sums[2]) - exponent(rho_new) > 33)  // (2^-33 = 1.2e-10)
+          stop = 4;
         else verdict();
       }
     }
