@@ -65,3 +65,31 @@ def test_batch_edge_data(count):
         out.append([c.populations() for c in m])
     for other in out[1:]:
         assert all(np.array_equal(a, b) for a, b in zip(out[0], other))
+
+
+@pytest.mark.parametrize("offset", [0, 4, 16])
+@pytest.mark.parametrize("shape,precision", [((33, 21), 32), ((130, 97), 64), ((517, 301), 32)])
+def test_every_byte_of_a_state_is_written(shape, precision, offset):
+    """Saved into buffers of two fills: a byte that keeps its fill in both was not
+    written, and those are the ones that the copies to host memory leave alone,
+    the padding between sections."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    lat = _lattice(*shape, precision)
+    ud = inputs.edge_array(*shape, 1.0, 1.0, 1.0, 1.0)
+    lat.substeps(12, 1, ud, ud)
+    nb = lat.state_bytes()
+    fills = (7, 200)
+    host = [lat.save(np.full(nb, v, np.uint8)) for v in fills]
+    dev = []
+    for v in fills:
+        room = torch.full((nb + 64,), v, dtype=torch.uint8, device="cuda")
+        lat.save(room[offset:offset + nb])
+        lat.synchronize()
+        got = room.cpu().numpy()
+        assert (got[:offset] == v).all() and (got[offset + nb:] == v).all()
+        dev.append(got[offset:offset + nb])
+    kept = [(a == fills[0]) & (b == fills[1]) for a, b in (host, dev)]
+    assert np.array_equal(*kept) and 0 < kept[0].sum() < 20 * 256
+    assert all(np.array_equal(a, b) for a, b in zip(host, dev))
