@@ -171,19 +171,21 @@ __device__ __forceinline__ void equilibrium(Real (&feq)[9], Real u, Real vx, Rea
 // only in the sign of 3 e.v; the rest population takes the remainder
 // f*_0 = (1 - k) u - sum_{i>0} f*_i, which is the same value in exact
 // arithmetic (sum_i f*_i = (1 - k) u) and keeps the stored populations
-// summing to the post-reaction mass in FP32.
+// summing to the post-reaction mass: the weights sum to 1 + 7.5e-9 in FP32 and
+// to 1 - 5.6e-17 in FP64, which would grow with every step.
 template <typename Real>
 __device__ __forceinline__ void collide(Real (&f)[9], Real u, Real vx, Real vy,
                                         const StepArgs<Real>& a, Real kr) {
   const Real omega = a.omega;
   if constexpr (sizeof(Real) == 8) {
     // FP64: the FP64 pipe bounds the step, so the form with the fewest FP64
-    // operations, 38 a node and 8 for u: the rest population in closed form
-    // (the weights sum to one to 1e-17), the weights taken into factors that
-    // the host forms (4.5 w = 1/2 and 1/8, 3 w = 1/3 and 1/12), each
-    // population two fused multiply-adds.  A ten-step call at 1024 x 1024 went
-    // from 1072 to 926 us by this form (43 operations before) and by shares
-    // without a division (kPerW).
+    // operations, 45 a node and 8 for u: the weights taken into factors that
+    // the host forms (4.5 w = 1/2 and 1/8, 3 w = 1/3 and 1/12), each moving
+    // population two fused multiply-adds, the remainder's sum as a tree.
+    // One pass of ten steps at 1024 x 1024 with its read-outs went from 1350 to
+    // 1100 us by this form and by shares without a division (kPerW).  The
+    // rest population in closed form saves 7 operations (1000 us), but then the
+    // mass drifts by up to 1.1e-16 of itself with every step.
     const Real x2 = vx * vx, y2 = vy * vy;
     const Real base = (Real)1 - (Real)1.5 * (x2 + y2);
     const Real us = u * (omega * base - kr);
@@ -191,7 +193,6 @@ __device__ __forceinline__ void collide(Real (&f)[9], Real u, Real vx, Real vy,
     const Real b1 = a.om_third * u, b5 = (Real)0.25 * b1;
     const Real s1 = (Real)w_of(1) * us, s5 = (Real)w_of(5) * us;
     const Real ne = vx + vy, nw = vy - vx;
-    f[0] = a.om1 * f[0] + (Real)w_of(0) * us;
     const Real t[4] = {a1 * x2 + s1, a1 * y2 + s1, a5 * (ne * ne) + s5, a5 * (nw * nw) + s5};
     const Real ev[4] = {vx, vy, ne, nw};
 #pragma unroll
@@ -201,6 +202,7 @@ __device__ __forceinline__ void collide(Real (&f)[9], Real u, Real vx, Real vy,
       f[i] = b * ev[p] + (a.om1 * f[i] + t[p]);
       f[o] = (a.om1 * f[o] + t[p]) - b * ev[p];
     }
+    f[0] = (u - kr * u) - (((f[1] + f[3]) + (f[2] + f[4])) + ((f[5] + f[7]) + (f[6] + f[8])));
     return;
   }
   const Real base = (Real)1 - (Real)1.5 * (vx * vx + vy * vy);
