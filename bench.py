@@ -41,12 +41,11 @@ METRIC = "LBM-ADE GLUPS & % HBM roofline (FP32 vs FP64); adjoint/forward time ra
 # the information content.)
 BYTES_FLUID = {32: 9 * 4 * 2 + 2 * 4 + 1, 64: 9 * 8 * 2 + 2 * 8 + 1}
 BYTES_SOLID = 1
-# FP64 arithmetic of the fused step per fluid node (an FMA counts 2): 8 adds
-# for u, 14 for the factors shared by all directions (v.v, 1 - omega, the
-# rest population's (1 - k) u, the e.v of the diagonals), 15 per opposite
-# pair (4 pairs).  The counters of the FP64 kernel show about 109 executed,
-# the rest being boundary code and idle lanes in blocks on a side.
-FLOPS_FLUID_FP64 = 82
+# FP64 arithmetic of the fused step per fluid node (an FMA counts 2), 53
+# operations: 8 adds for u, 26 for the factors shared by all directions and the
+# four pairs' symmetric parts, 8 per opposite pair (4 pairs), 10 for the rest
+# population's remainder.
+FLOPS_FLUID_FP64 = 76
 FP64_PEAK_GFLOPS = 1250.0  # nominal dense FP64 of one GB300
 
 
@@ -533,8 +532,8 @@ def main():
                                  "flops_per_fluid_node": FLOPS_FLUID_FP64}}
 
     # ---- the same workload with maximum-entropy pore walls ---------------------
-    # both precisions of the wall solve: the Lagrange multiplier by Newton's
-    # method in FP64 ("maxent") and in FP32 ("maxent_lattice")
+    # both precisions of the wall solve: beyond FP32 ("maxent": double-float, in
+    # FP64 at the ends of its range) and Newton's method in FP32 ("maxent_lattice")
     walls = None
     if args.walls_steps > 0:
         walls = {}
@@ -559,7 +558,7 @@ def main():
             walls[mode] = {
                 "value": world * nodes * args.walls_steps / (msw / 1e3) / 1e9,
                 "unit": "GLUPS", "steps": args.walls_steps,
-                "newton_precision": "f64" if mode == "maxent" else "f32",
+                "newton_precision": "f32x2" if mode == "maxent" else "f32",
                 "ms_per_step": msw / args.walls_steps,
                 "kernel_ms_per_launch": sw_ms / max(sw_n, 1),
                 "bc_infeasible": dw["bc_infeasible"], "newton_fail": dw["newton_fail"],

@@ -41,7 +41,10 @@ __device__ __forceinline__ void move_as(char* dst, const char* src, size_t len) 
 // whose separate copies took about 5 us each (2 of work, 3 between two of
 // them).  Ten substeps of a 256 x 64 channel with restore and trace went from 139
 // to 119 us, 50 of a dissolving 512 x 512 block from 653 to 552, 25 of 24 lattices
-// together, with 72 pieces of edge data, from 2.58 to 2.21 ms.
+// together, with 72 pieces of edge data, from 2.58 to 2.21 ms.  Large states
+// gain too: saved and restored, 1024 x 1024 nodes with mineral (73 MB) took 98
+// and 103 us as separate copies, 28 and 43 this way; 4096 x 4096 (1.15 GB)
+// 435 and 427, now 343 and 388.
 __global__ void __launch_bounds__(kCopyThreads) k_copy_list(const __grid_constant__ CopyArgs a) {
   if (blockIdx.x == 0 && (int)threadIdx.x < a.head_bytes) a.head_dst[threadIdx.x] = a.head[threadIdx.x];
   if (a.n == 0) return;  // the head alone

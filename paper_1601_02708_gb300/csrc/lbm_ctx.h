@@ -217,8 +217,8 @@ inline lbm::StepArgs<Real> step_args(lbm_ctx* c, double frac) {
 }
 
 // Template argument kWalls of the step kernels for the context's wall mode:
-// 0 without maximum-entropy walls, 2 for FP64 Newton solves on the FP32
-// lattice, 1 for solves in the lattice's own precision.
+// 0 without maximum-entropy walls, 2 for solves beyond the FP32 lattice's
+// precision (LBM_WALL_MAXENT there), 1 for solves in the lattice's own.
 inline int walls_variant(const lbm_ctx* c) {
   if (c->wall_mode == LBM_WALL_BOUNCE) return 0;
   return (c->wall_mode == LBM_WALL_MAXENT && c->esize == 4) ? 2 : 1;

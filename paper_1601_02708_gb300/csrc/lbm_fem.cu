@@ -20,7 +20,7 @@
 // solves A x = B d^n (+ prescribed values) by Jacobi-preconditioned
 // BiCGSTAB in FP64 inside one cooperative launch, the host reading the outcome
 // once per step: by tiles held in shared memory where the mesh fits (about
-// 200,000 nodes, k_bicgstab_tile), else over the nodes in global memory with
+// 160,000 nodes, k_bicgstab_tile), else over the nodes in global memory with
 // grid-wide barriers between the phases (k_bicgstab).  Sums are the same in
 // every block and in every run.  A
 // solve starts from the last converged solution (the previous Schwarz
@@ -405,7 +405,10 @@ constexpr int kTileVals = 5;        // values an exchange carries at most
 constexpr int kTileSlot = 8;        // 16-byte words from block to block: one 128-byte line
 constexpr int kTileMaxBlocks = 256;  // at most eight per polling lane
 // 12 warps: one node a thread of the 286-node tiles of a 400 x 100 mesh and of
-// their rings (with 8 the few nodes left over cost a second pass)
+// their rings (with 8 the few nodes left over cost a second pass).  A step of
+// 23 iterations with 8, 12 and 16 warps, us: 451 nodes 227, 229, 256; 20,301
+// 277, 279, 326; 40,501 339, 314, 354; 60,501 363, 390, 408; 100,651 433, 421,
+// 485; 135,751 469, 468, 546.
 constexpr int kTileThreads = 384;
 constexpr unsigned long long kTileWaitNs = 2000000000ull;  // 2 s
 
@@ -882,7 +885,10 @@ namespace {
 // Tile of k_bicgstab_tile for the mesh: the one whose block does the least
 // FP64 work per iteration, in warp instructions (6 a ring entry and 26 an own
 // node, and about 80 + 6 (blocks / 32 + 5) for the sums), among those whose
-// blocks are at most one per SM and fit its shared memory.  Larger meshes keep
+// blocks are at most one per SM and fit its shared memory, which is the better
+// solve wherever it fits: a step of 23 iterations takes 229 us instead of 266
+// with 451 nodes, 262 instead of 703 with 5,151, 279 instead of 687 with 20,301,
+// 390 instead of 1008 with 60,501, 468 instead of 1217 with 135,751.  Larger meshes keep
 // the cooperative solve over all nodes (tiles = 0).
 constexpr size_t kTileSmem = 200 * 1024;
 void pick_tile(lbm_fem* f, int sms) {

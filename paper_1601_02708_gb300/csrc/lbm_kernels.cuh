@@ -42,8 +42,8 @@ constexpr int kBY = 8;   // generic kernel: rows per block
 // 4096^2 with 32 x 8 blocks (32 x 16 blocks: 237 us), with the same warps
 // active and the same DRAM bytes but DRAM busier (61 against 59% of peak in
 // a 2048^2 capture).  FP64: 8, since its interior blocks pack their
-// updating nodes into the first lanes, which larger blocks do better (1.40
-// against 1.46 ms at 32 x 4).
+// updating nodes into the first lanes, which larger blocks do better (4096^2, with
+// 82 flops a node instead of 76: 1.40 ms, 1.46 at 32 x 4 and 1.60 at 32 x 2).
 template <typename Real>
 __host__ __device__ constexpr int step_rows() {
   return sizeof(Real) == 4 ? 2 : 8;
@@ -51,8 +51,13 @@ __host__ __device__ constexpr int step_rows() {
 // FP64 lattices of fewer than five 32 x 8 blocks per SM run 32 x 2: there the
 // step is as long as the SM with the most warps keeps its FP64 pipe, and small
 // blocks spread (a 256 x 64 lattice: 4 warps on every SM, not 8 on 64 of 152):
-// 8.1 -> 5.7 us a substep there, 13.0 -> 10.5 at 331 x 203 with pores, 21.2 ->
-// 18.1 at 512 x 256, whose 512 blocks of 32 x 8 are three or four to an SM.
+// 8.8 -> 6.4 us a substep there, 13.6 -> 11.9 at 331 x 203 with pores, 22.9 ->
+// 18.7 at 512 x 256, whose 512 blocks of 32 x 8 are three or four to an SM.
+// With pores the shapes are even at five and six blocks an SM (24.5 and 24.1 us
+// at 512 x 384, 27.3 and 27.4 at 640 x 384) and 32 x 8, which packs its fluid
+// nodes, is ahead from eight on (31.3 against 33.0 at 600 x 500, 37.7 against
+// 39.0 at 768 x 512, 84.2 against 92.1 at 1024 x 1024); without pores 32 x 2
+// gains 1.5 us at five and 1.7 (of 118) at 27.
 constexpr int kSmallRows = 2;
 
 template <typename Real>
@@ -305,10 +310,12 @@ __device__ __forceinline__ void store_share(const StepArgs<Real>& a, long long n
 // from every side, so no pull leaves the lattice, no ghost image exists and
 // the node is not on the outlet; the boundary code is then compiled out.
 // kSolve: the node may lie on a non-periodic side, whose populations pulled
-// from outside are set by the maximum-entropy conditions (in FP64 on either
-// lattice); callers that route those nodes elsewhere compile the solves out.
+// from outside are set by the maximum-entropy conditions (from FP64 edge data,
+// in double-float on the FP32 lattice and FP64 on the FP64 one); callers that
+// route those nodes elsewhere compile the solves out.
 // kWalls: 0, the kernel carries no wall code; 1, maximum-entropy pore walls
-// (when a.wall_maxent) solved in the lattice's precision; 2, solved in FP64.
+// (when a.wall_maxent) solved in the lattice's precision; 2, to better than
+// FP32 populations hold (maxent_wall).
 // kLight: the node's inputs are cheap to read (a shared-memory tile), so a
 // solid lane runs the fluid lanes' arithmetic on its (finite) inputs and
 // discards it: the warp takes one path and issues one set of stores, where

@@ -10,9 +10,9 @@
 // generic kernel, and store f* with coalesced row writes.  (The update is
 // bound by the consumers' instruction latency, so the tile is sized for as
 // many consumer warps as the register file holds.)  The nodes on
-// non-periodic sides, whose boundary solves run in FP64 (slow on this part),
-// are left to one boundary warp per CTA that reads them from global memory
-// beside the pipeline, so no consumer warp waits on the FP64 pipe.  Every
+// non-periodic sides, whose boundary solves are long chains (double-float, from
+// FP64 edge data), are left to one boundary warp per CTA that reads them from
+// global memory beside the pipeline, so no consumer warp waits for them.  Every
 // wait on an mbarrier has an iteration limit: on expiry the CTA records a
 // status, drains its copies in flight (again with a limit) and returns.
 #pragma once

@@ -16,9 +16,9 @@ from ._lib import Diag, LBMError, Params, check
 
 PERIODIC, DIRICHLET, NEUMANN = 0, 1, 2
 REACT_NONE, REACT_SURFACE, REACT_BULK = 0, 1, 2
-# lbm_wall_mode: halfway bounce-back; zero-flux maximum entropy with the
-# Newton solve in FP64 ("maxent") or in the lattice's own precision
-# ("maxent_lattice", FP32 on an FP32 lattice)
+# lbm_wall_mode: halfway bounce-back; zero-flux maximum entropy solved to
+# better than FP32 populations hold ("maxent": double-float or FP64) or in the
+# lattice's own precision ("maxent_lattice", FP32 on an FP32 lattice)
 WALLS = {"bounce": 0, "maxent": 1, "maxent_lattice": 2}
 
 
@@ -92,12 +92,12 @@ class LBM:
     (PERIODIC, DIRICHLET or NEUMANN), solid mask, advection velocity
     [2, ny, nx], initial concentration, and the first-order reaction
     (``react_mode``, ``k`` or ``k_field``, ``dissolution``, ``mineral``).
-    ``precision`` 32 runs FP32 populations with FP64 boundary solves and
-    sums; 64 runs FP64 throughout.  ``walls`` treats the pore walls by
-    halfway bounce-back ("bounce") or as zero-flux boundaries of the
-    maximum-entropy kind (Sec. 4.1.1 (b)) with the Lagrange multiplier's
-    Newton solve in FP64 ("maxent") or in the lattice's precision
-    ("maxent_lattice").
+    ``precision`` 32 runs FP32 populations with boundary solves in
+    double-float from FP64 edge data and FP64 sums; 64 runs FP64 throughout.
+    ``walls`` treats the pore walls by halfway bounce-back ("bounce") or as
+    zero-flux boundaries of the maximum-entropy kind (Sec. 4.1.1 (b)) solved
+    to better than FP32 populations hold ("maxent") or in the lattice's
+    precision ("maxent_lattice").
     """
 
     def __init__(self, nx, ny, tau, edges=(PERIODIC,) * 4, precision=32,
