@@ -208,14 +208,17 @@ __device__ __forceinline__ int maxent_neumann_general(Real (&f)[9], unsigned unk
 // on this part and the general form has some thirty in a row), and with it the
 // step of a small lattice, whose boundary nodes are one round of one warp.
 // FP32 lattice: the sums and the product run in double-float (sums exact to
-// 2^-48 of the largest term) on the FP32 pipe.  The general form keeps every
-// case this one does not hold: other unknown sets, Neumann corners, values
-// outside 1e-24 .. 1e30 (the low parts leave FP32's range), and differences a
-// thousand times smaller than their terms.
-// FP64 lattice: the same in FP64, the sum as a tree.
+// 2^-48 of the largest term) on the FP32 pipe.  What this does not hold goes to
+// the FP64 form: values outside 1e-24 .. 1e30 (the low parts leave FP32's range)
+// and differences a thousand times smaller than their terms.
+// FP64 lattice: the same in FP64, the sum as a tree, seven operations in a row.
+// The general form keeps other unknown sets and Neumann corners.
 // Ten substeps of a 256 x 64 channel with restore and trace: 145 -> 139 us; one
 // gradient over 500 steps at 512 x 512, whose reverse steps transpose the same
 // solves: 10.2 -> 8.3 ms; a coarse step of the plain hybrid in FP64: 724 -> 700.
+// A substep at 512 x 512: general form alone 6.1 us, FP64 form 5.85, double-float
+// 5.6, and 6.15 with a boundary node or two beyond its range (6.9 when those took
+// the general form).
 constexpr float kEdgeLow = 1e-24f, kEdgeHigh = 1e30f, kEdgeCancel = 1e-3f;
 
 struct EdgeSum {  // hi + lo, not normalised
@@ -252,6 +255,39 @@ __device__ __forceinline__ int set_weight36(unsigned m) {
   return 4 * __popc(m & 0x1Eu) + __popc(m & 0x1E0u);
 }
 
+// The FP64 form, the sums as trees: weight 36 W_U = c is 6 or 11; on a side, whose
+// unknowns all have e.n = -1.
+template <typename Real>
+__device__ __forceinline__ bool dirichlet_tree(Real (&f)[9], unsigned unknown, double up, int c) {
+  double k[9];
+#pragma unroll
+  for (int i = 0; i < 9; ++i) k[i] = unknown & (1u << i) ? 0.0 : (double)f[i];
+  const double known = (((k[0] + k[1]) + (k[2] + k[3])) + ((k[4] + k[5]) + (k[6] + k[7]))) + k[8];
+  const double rest = up - known;
+  const double g = rest * (c == 6 ? 1.0 / 6 : 1.0 / 11), g4 = 4.0 * g;
+#pragma unroll
+  for (int i = 1; i < 9; ++i)
+    if (unknown & (1u << i)) f[i] = (Real)(i < 5 ? g4 : g);
+  return rest < 0.0;
+}
+template <typename Real>
+__device__ __forceinline__ int neumann_tree(Real (&f)[9], unsigned unknown, int sx, int sy, double q) {
+  double k[9];
+#pragma unroll
+  for (int i = 1; i < 9; ++i) {
+    const int d = cx_of(i) * sx + cy_of(i) * sy;
+    k[i] = unknown & (1u << i) ? 0.0 : d > 0 ? (double)f[i] : d < 0 ? -(double)f[i] : 0.0;
+  }
+  const double out = ((k[1] + k[2]) + (k[3] + k[4])) + ((k[5] + k[6]) + (k[7] + k[8]));
+  const double S = out - q;
+  const bool root = S > 0.0;
+  const double g = S * (1.0 / 6), g4 = 4.0 * g;
+#pragma unroll
+  for (int i = 1; i < 9; ++i)
+    if (unknown & (1u << i)) f[i] = root ? (Real)(i < 5 ? g4 : g) : (Real)0;
+  return root ? kNeuRoot : S < 0.0 ? kNeuInfeasible : kNeuZero;
+}
+
 __device__ __forceinline__ bool maxent_dirichlet(float (&f)[9], unsigned unknown, double up) {
   EdgeSum rest = edge_split(up), known;
   float most = fabsf(rest.hi);
@@ -279,22 +315,12 @@ __device__ __forceinline__ bool maxent_dirichlet(float (&f)[9], unsigned unknown
       if (unknown & (1u << i)) f[i] = 0.f;
     return false;
   }
-  return maxent_dirichlet_general(f, unknown, up);
+  return c == 6 || c == 11 ? dirichlet_tree(f, unknown, up, c) : maxent_dirichlet_general(f, unknown, up);
 }
 
 __device__ __forceinline__ bool maxent_dirichlet(double (&f)[9], unsigned unknown, double up) {
   const int c = set_weight36(unknown);
-  if (c != 6 && c != 11) return maxent_dirichlet_general(f, unknown, up);
-  double k[9];
-#pragma unroll
-  for (int i = 0; i < 9; ++i) k[i] = unknown & (1u << i) ? 0.0 : f[i];
-  const double known = (((k[0] + k[1]) + (k[2] + k[3])) + ((k[4] + k[5]) + (k[6] + k[7]))) + k[8];
-  const double rest = up - known;
-  const double g = rest * (c == 6 ? 1.0 / 6 : 1.0 / 11), g4 = 4.0 * g;
-#pragma unroll
-  for (int i = 1; i < 9; ++i)
-    if (unknown & (1u << i)) f[i] = i < 5 ? g4 : g;
-  return rest < 0.0;
+  return c == 6 || c == 11 ? dirichlet_tree(f, unknown, up, c) : maxent_dirichlet_general(f, unknown, up);
 }
 
 __device__ __forceinline__ int maxent_neumann(float (&f)[9], unsigned unknown, int sx, int sy,
@@ -330,6 +356,7 @@ __device__ __forceinline__ int maxent_neumann(float (&f)[9], unsigned unknown, i
         if (unknown & (1u << i)) f[i] = 0.f;
       return kNeuZero;
     }
+    return neumann_tree(f, unknown, sx, sy, q);
   }
   return maxent_neumann_general(f, unknown, sx, sy, q, fbb);
 }
@@ -338,20 +365,7 @@ __device__ __forceinline__ int maxent_neumann(double (&f)[9], unsigned unknown, 
                                               double q, const double (&fbb)[9]) {
   if ((sx != 0 && sy != 0) || set_weight36(unknown) != 6)
     return maxent_neumann_general(f, unknown, sx, sy, q, fbb);
-  double k[9];
-#pragma unroll
-  for (int i = 1; i < 9; ++i) {
-    const int d = cx_of(i) * sx + cy_of(i) * sy;
-    k[i] = unknown & (1u << i) ? 0.0 : d > 0 ? f[i] : d < 0 ? -f[i] : 0.0;
-  }
-  const double out = ((k[1] + k[2]) + (k[3] + k[4])) + ((k[5] + k[6]) + (k[7] + k[8]));
-  const double S = out - q;
-  const bool root = S > 0.0;
-  const double g = S * (1.0 / 6), g4 = 4.0 * g;
-#pragma unroll
-  for (int i = 1; i < 9; ++i)
-    if (unknown & (1u << i)) f[i] = root ? (i < 5 ? g4 : g) : 0.0;
-  return root ? kNeuRoot : S < 0.0 ? kNeuInfeasible : kNeuZero;
+  return neumann_tree(f, unknown, sx, sy, q);
 }
 
 // Boundary kind of an edge node (x, y) whose unknown set is not empty:
