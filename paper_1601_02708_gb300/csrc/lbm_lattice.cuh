@@ -428,6 +428,9 @@ __device__ int maxent_wall_general(Real (&f)[9], unsigned solid) {
       my -= w36 * cy_of(i);
     }
   if (mx == 0 && my == 0) return kWallSet;
+  // FP32 populations in an FP64 solve: integer multiples of them, summed before
+  // the normal is scaled, so that a flux that cancels keeps its sign
+  constexpr bool kExact = sizeof(S) == 8 && sizeof(Real) == 4;
   const S inv = (S)1 / sqrt((S)(mx * mx + my * my));
   const S nx = (S)mx * inv, ny = (S)my * inv;
   S a[9], R = (S)0, s1 = (S)0, s2 = (S)0;
@@ -439,10 +442,13 @@ __device__ int maxent_wall_general(Real (&f)[9], unsigned solid) {
       neg |= 1u << i;
       s1 -= (S)w_of(i) * a[i];
       s2 += (S)w_of(i) * a[i] * a[i];
+    } else if (kExact) {
+      R -= (S)(cx_of(i) * mx + cy_of(i) * my) * (S)f[i];
     } else {
       R -= a[i] * (S)f[i];
     }
   }
+  if (kExact) R *= inv;
   if (!neg) return kWallSet;
   if (!(R < (S)0)) {
 #pragma unroll
@@ -711,14 +717,15 @@ __device__ __forceinline__ bool wall_root(const WallPoly& w, double T, WallValue
 // The wall solve of a step.  The FP64 solve takes the polynomial form: with
 // its exponentials in FP64 (1/64 of the FP32 rate on this part, and every warp
 // with one wall node pays for 32) the solve took nearly all of the step's time,
-// 480 us a step at 1200 x 900 with FP32 populations; with one double-float
-// evaluation on the FP32 pipe the step takes 28 to 44, by the data.  The
+// 521 us a step at 1200 x 900 with FP32 populations; with one double-float
+// evaluation on the FP32 pipe the step takes 42 (bounce-back walls: 12.5).  The
 // general form, in logarithms, takes over where T is outside 1e-24 .. 1e24 for
 // FP32 populations (there the low parts of the FP32 pairs or the powers of t
 // leave FP32's range), outside 1e-34 .. 1e34 for FP64 ones (the range of the FP32
-// start), or where the start did not converge; it works on a copy of f, so that
-// the usual path keeps f in registers.  A lattice that starts empty has many
-// such walls ahead of its front: there a step takes 83 us instead of 222.
+// start), where a flux of FP32 populations cancels, or where the start did not
+// converge; it works on a copy of f, so that the usual path keeps f in
+// registers.  A lattice that starts empty has many such walls ahead of its
+// front: there a step takes 56 us instead of 184.
 template <typename S, typename Real>
 __device__ __noinline__ int maxent_wall_rare(Real* f, unsigned solid) {
   Real g[9];
@@ -728,18 +735,6 @@ __device__ __noinline__ int maxent_wall_rare(Real* f, unsigned solid) {
 #pragma unroll
   for (int i = 0; i < 9; ++i) f[i] = g[i];
   return r;
-}
-
-// sum_{others} (e_j.m) f_j in FP64 (out of line: a wall whose flux cancels is rare)
-static __device__ __noinline__ double wall_flux(float f1, float f2, float f3, float f4, float f5,
-                                                float f6, float f7, float f8, unsigned neg, int mx,
-                                                int my) {
-  const float f[9] = {0.f, f1, f2, f3, f4, f5, f6, f7, f8};
-  double T = 0.0;
-#pragma unroll
-  for (int i = 1; i < 9; ++i)
-    if (!(neg & (1u << i))) T += (double)(cx_of(i) * mx + cy_of(i) * my) * (double)f[i];
-  return T;
 }
 
 template <typename S, typename Real>
@@ -782,18 +777,12 @@ __device__ __forceinline__ int maxent_wall(Real (&f)[9], unsigned solid) {
       }
     }
     if (!neg) return kWallSet;
-    Df Td = df_norm(Th, Tl);
-    if constexpr (sizeof(Real) == 4) {
-      // the pair holds the sum to 2^-48 of its largest term: where less than a
-      // thousandth of that is left (or a product overflows) it is summed in FP64
-      if (most > 0.f && !(fabsf(Td.hi) > kEdgeCancel * most && most < kEdgeHigh)) {
-        T = wall_flux(f[1], f[2], f[3], f[4], f[5], f[6], f[7], f[8], neg, mx, my);
-        Td.hi = (float)T;
-        Td.lo = (float)(T - (double)Td.hi);
-      }
-    }
+    const Df Td = df_norm(Th, Tl);
     const Real size = sizeof(Real) == 8 ? (Real)T : (Real)Td.hi;
-    if (!(size > (Real)0)) {
+    // the pair holds the sum to 2^-48 of its largest term: where less than a
+    // thousandth of that is left (or a product overflows) the rare form sums it
+    const Real least = sizeof(Real) == 8 ? (Real)0 : (Real)(kEdgeCancel * most);
+    if (!(size >= -least) || (size == (Real)0 && least == (Real)0)) {
 #pragma unroll
       for (int i = 1; i < 9; ++i)
         if (neg & (1u << i)) f[i] = (Real)0;
@@ -801,7 +790,7 @@ __device__ __forceinline__ int maxent_wall(Real (&f)[9], unsigned solid) {
     }
     WallValues<Real> v;
     constexpr double kLow = sizeof(Real) == 8 ? 1e-34 : 1e-24;
-    bool ok = size > (Real)kLow && size < (Real)(1.0 / kLow);
+    bool ok = size > (Real)kLow && size < (Real)(1.0 / kLow) && size > least;
     if (ok) {
       if constexpr (sizeof(Real) == 8) ok = wall_root(w, T, v);
       else ok = wall_root(w, Td, v);
