@@ -203,15 +203,15 @@ lbm_status lbm_min_population(lbm_ctx* c, double* out);
  * neighbours, n = -sum w_i e_i over those directions (normalised); unknowns
  * with e_i.n >= 0 keep bounce-back, as does a node where the sum cancels.
  * On an FP32 lattice the flux of the known populations is summed and the root
- * found in double-float (the flux in FP64 where it cancels to less than a
- * thousandth of its largest term, all of it in FP64 below 1e-24 and above
- * 1e24): the populations are within 1.1e-9 relative of the root's (1.8e-9
- * where all is in FP64) and rounded to FP32 once.  On an FP64 lattice it runs
+ * found in double-float, or in FP64 where the flux cancels to less than a
+ * thousandth of its largest term, is below 1e-24 or above 1e24: the populations
+ * are within 1.1e-9 relative of the root's (FP64: 1.8e-9, its stopping rule on
+ * an FP32 lattice) and rounded to FP32 once.  On an FP64 lattice it runs
  * in FP64 to rounding.  LBM_WALL_MAXENT_LATTICE: on an FP32 lattice Newton's
  * method in FP32 (tolerance 5e-7), which is faster: a 1200 x 900 pore lattice
- * steps in 20 us with it, in 28 to 83 us with LBM_WALL_MAXENT (the most where
- * fluxes are below 1e-24, ahead of a front) and in 13 us with bounce-back;
- * on an FP64 lattice the same as LBM_WALL_MAXENT.
+ * steps in 19 to 32 us with it, in 42 to 56 us with LBM_WALL_MAXENT (the most
+ * where fluxes are below 1e-24, ahead of a front) and in 12.5 us with
+ * bounce-back; on an FP64 lattice the same as LBM_WALL_MAXENT.
  * Solves with no root set their unknowns to zero and count in
  * lbm_diag.bc_infeasible; solves short of the tolerance count in
  * lbm_diag.newton_fail.  The adjoint (lbm_adjoint) covers bounce-back walls
