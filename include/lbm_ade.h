@@ -520,7 +520,8 @@ const char* lbm_mass_noalloc_error(void);
  *
  * A message of phase 0 carries the three populations that stream across the
  * side from the boundary row and, with dissolution, that row's reaction
- * shares; phase 1 carries the boundary row's solid and turning-fluid flags,
+ * shares (on an FP32 lattice with a rate field its rates too); phase 1 carries
+ * the boundary row's solid and turning-fluid flags,
  * from which the receiver sets its links across the cut and lists the solid
  * nodes a neighbour's flip exposed.  lbm_halo_bytes gives a message's size
  * (the same for both sides).  Buffers are device memory of the slab's

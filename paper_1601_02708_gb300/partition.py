@@ -7,7 +7,8 @@ ghost row beyond a shared side.  Every step of the method runs in the
 library: ``lbm_step_stream`` and ``lbm_step_dissolve`` are the two halves of
 a time step, ``lbm_halo_pack`` / ``lbm_halo_unpack`` build and apply the two
 messages each shared side carries per step (phase 0 after the fused step:
-the populations that stream across and the reaction shares; phase 1 after
+the populations that stream across and the reaction shares (with the rates of
+an FP32 lattice's rate field); phase 1 after
 the dissolution pass: the boundary row's solid flags).  This module only
 sequences the calls and moves the messages: between slabs held by one
 process (``LocalExchange``, device-to-device copies -- several slabs on one
